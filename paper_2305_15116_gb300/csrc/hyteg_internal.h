@@ -67,6 +67,15 @@ struct LevelDev {
   int64_t* if_flat_base = nullptr;
   int* if_rest = nullptr;
   int n_if_rest = 0;
+  // 3D: interface work list of the one-launch apply, int4 (prim, first
+  // point, points, lanes per point)
+  int4* if3 = nullptr;
+  int n_if3 = 0;
+  // 3D, small vectors: one thread per macro-interior point, from the table of
+  // the macro's interior points (slot, row length | slice side << 16)
+  bool direct3 = false;
+  int2* pts3 = nullptr;
+  int n_pts3 = 0;
   // 3D row-kernel work list: int4 (x0, y0, y1, z): lattice columns x0-1..x0+30
   // (x0..x0+29 written), rows y0..y1-1 of slice z of one macro
   int4* r3_tiles = nullptr;
@@ -341,6 +350,18 @@ cudaError_t slab3d_prepare();
 // the slab kernel over an explicit work list (the autotuner's candidates)
 cudaError_t launch_slab3d_items(int dtype, const LevelDev& L, const int4* items, int n_items, const void* x,
                                 void* y, cudaStream_t s);
+// Levels whose vectors the direct 3D kernel takes (LevelDev::direct3): up to
+// 2^21 slots it is faster than the slab kernel and its interface launch in
+// every element type (us per apply, direct / slab + interface; float64, fp32,
+// native: 35k slots 11.0 / 21.2, 10.9 / 13.3; 0.47M slots 11.1 / 48.1,
+// 10.9 / 28.7, 14.0 / 78.7; 1.9M slots 37.8 / 62.5, 14.5 / 31.1, 52.6 / 102;
+// at 18M slots 337 / 298, 144 / 131).
+constexpr int kDirect3MaxN = 64;
+constexpr int64_t kDirect3MaxSlots = int64_t(1) << 21;
+// the direct 3D kernel of several meshes in one launch, interface step
+// included (partial: every interface copy keeps its own macro's partial row)
+cudaError_t launch_direct3d_group(int dtype, bool partial, const Mesh* const* ms, const int* levels,
+                                  const void* const* xs, void* const* ys, int count, cudaStream_t s);
 cudaError_t launch_row3d(int dtype, const LevelDev& L, int64_t n_cells, const void* x, void* y, cudaStream_t s);
 cudaError_t build_iface_slots(const Mesh& m, const LevelDev& L, cudaStream_t s);
 cudaError_t launch_interface_reduce(int dtype, const Mesh& m, int level, const void* x, void* y, cudaStream_t s);

@@ -335,6 +335,17 @@ cudaError_t launch_apply(const Mesh& m, int level, int dtype, const void* x, voi
     }
     return e;
   }
+  if (L.direct3) {  // small vectors: one launch
+    *what = "3D apply kernel";
+    const Mesh* mp = &m;
+    e = launch_direct3d_group(dtype, false, &mp, &level, &x, &y, 1, s);
+    if (e != cudaSuccess) return e;
+    if (ev_mid) {
+      *what = "cudaEventRecord";
+      e = cudaEventRecord(ev_mid, s);
+    }
+    return e;
+  }
   // 3D: the slab kernel (n <= 64: whole slices in shared memory) or the row
   // kernel (larger levels) writes every slot, partial rows at macro
   // boundaries included; the interface step then reduces the copies
@@ -358,8 +369,12 @@ cudaError_t launch_apply_partial(const Mesh& m, int level, int dtype, const void
     *what = "2D apply kernel (partial rows)";
     return launch_apply2d_partial(dtype, m, L, x, y, s);
   }
-  // 3D: the slab or row kernel writes the partial rows; no reduction
+  // 3D: the macro kernel leaves the partial rows; no reduction
   *what = "3D kernel";
+  if (L.direct3) {
+    const Mesh* mp = &m;
+    return launch_direct3d_group(dtype, true, &mp, &level, &x, &y, 1, s);
+  }
   return L.n_slabs > 0 ? launch_slab3d(dtype, L, x, y, s) : launch_row3d(dtype, L, m.n_cells, x, y, s);
 }
 

@@ -321,6 +321,8 @@ void free_level(const Mesh& m, LevelDev& L) {
   dev_free(m, L.slabs);
   for (int t = 0; t < 4; ++t) dev_free(m, L.slabs_dt[t]);
   dev_free(m, L.r3_tiles);
+  dev_free(m, L.pts3);
+  dev_free(m, L.if3);
   dev_free(m, L.if_slots);
   dev_free(m, L.if_item_base);
   dev_free(m, L.if_pairs);
@@ -580,6 +582,37 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     }
     L.n_r3_tiles = int(r3.size());
     if (!(err = upload(m, &L.r3_tiles, r3)).empty()) return err;
+  }
+  if (d == 3) {
+    // interface work list of the 3D apply (iface3d.cuh): (prim, first point,
+    // points, lanes per point), at most 128 threads per item
+    std::vector<int4> if3;
+    for (size_t p = 0; p < m.prims.size(); ++p) {
+      const Prim& pr = m.prims[p];
+      const int64_t np = pr.type == 0 ? 1 : pr.type == 1 ? n - 1 : int64_t(n - 1) * (n - 2) / 2;
+      int lanes = 1;
+      if (pr.inc_count > 2 && pr.inc_count <= 32 && !pr.boundary)
+        while (lanes < pr.inc_count) lanes *= 2;
+      const int per = 128 / lanes;
+      for (int64_t t = 0; t < np; t += per)
+        if3.push_back(make_int4(int(p), int(t), int(std::min<int64_t>(per, np - t)), lanes));
+    }
+    L.n_if3 = int(if3.size());
+    if (!(err = upload(m, &L.if3, if3)).empty()) return err;
+    L.direct3 = n <= kDirect3MaxN && L.slots_per_macro * m.n_cells <= kDirect3MaxSlots;
+    if (L.direct3) {  // the macro-interior points in slot order: (slot, A | M << 16)
+      std::vector<int2> pts;
+      int slot = 0;
+      for (int z = 0; z <= n; ++z)
+        for (int y = 0; y <= n - z; ++y)
+          for (int x = 0; x <= n - z - y; ++x, ++slot)
+            if (x > 0 && y > 0 && z > 0 && x + y + z < n) {
+              const int M = n + 1 - z;
+              pts.push_back(make_int2(slot, (M - y) | (M << 16)));
+            }
+      L.n_pts3 = int(pts.size());
+      if (!(err = upload(m, &L.pts3, pts)).empty()) return err;
+    }
   }
   if (d == 2) return build_p2_level(m, level, L);
   return "";

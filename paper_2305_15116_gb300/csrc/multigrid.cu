@@ -775,8 +775,26 @@ cudaError_t apply_g(Mesh* const* ms, int cnt, int l, int dtype, const void* cons
     if (ms[0]->dim == 2) {
       HY_TRY(launch_apply2d_batch(dt, mm.data(), lv.data(), xx.data(), yy.data(), k, s));
     } else {
-      HY_TRY(launch_slab3d_group(dt, mm.data(), lv.data(), xx.data(), yy.data(), k, s));
-      HY_TRY(launch_interface_reduce_group(dt, mm.data(), lv.data(), xx.data(), yy.data(), k, s));
+      // small vectors in one launch, the others with their interface step after it
+      for (int direct = 0; direct < 2; ++direct) {
+        std::vector<const Mesh*> md;
+        std::vector<const void*> xd;
+        std::vector<void*> yd;
+        for (int i = 0; i < k; ++i) {
+          if (int(mm[i]->levels[l].direct3) != direct) continue;
+          md.push_back(mm[i]);
+          xd.push_back(xx[i]);
+          yd.push_back(yy[i]);
+        }
+        if (md.empty()) continue;
+        const int kd = int(md.size());
+        if (direct) {
+          HY_TRY(launch_direct3d_group(dt, false, md.data(), lv.data(), xd.data(), yd.data(), kd, s));
+        } else {
+          HY_TRY(launch_slab3d_group(dt, md.data(), lv.data(), xd.data(), yd.data(), kd, s));
+          HY_TRY(launch_interface_reduce_group(dt, md.data(), lv.data(), xd.data(), yd.data(), kd, s));
+        }
+      }
     }
   }
   return cudaSuccess;
