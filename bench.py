@@ -169,21 +169,15 @@ def setup(name, device, dtype_code, level=None):
     interior = coarse.n_cells * ((n - 1) * (n - 2) // 2 if coarse.dim == 2 else (n - 1) * (n - 2) * (n - 3) // 6)
     slab = True  # every apply kernel writes every slot (interface copies included)
     # the library's kernel launches per apply: 2D one (macro interiors and
-    # interface points together); 3D the slab kernel (or the row kernel and
-    # its row-end companion) and the interface reduction; P2 the row and
-    # boundary kernels and the vertex and edge reductions
-    if p2:
-        launches = 4
-    elif coarse.dim == 2:
-        launches = 1
-    else:
-        launches = 2 if n <= 64 else 3
+    # interface points together), 3D one likewise; P2 the row and boundary
+    # kernels and the vertex and edge reductions
+    launches = 4 if p2 else 1
     if p2:
         kernel = "k_p2_apply"
         raw = lambda l, c, xp, yp, sp: M.p2_apply_timed(l, c, xp, yp, sp, 0, 0, 0)
         timed = M.p2_apply_timed
     else:
-        kernel = "k_interior2d" if coarse.dim == 2 else ("k_slab3d" if n <= 64 else "k_row3d")
+        kernel = "k_interior2d" if coarse.dim == 2 else "apply3d"
         raw, timed = M.apply_raw, M.apply_timed
     return dict(M=M, L=L, ns=ns, ng=ng, xs=xs, ys=ys, smap=smap, x_global=x, coarse=coarse,
                 interior=interior, elem=4 if dtype_code == H.F32 else 8, code=dtype_code, launches=launches,
@@ -307,8 +301,8 @@ def batched_small(w, count, stream, reps=50):
 
 def interior_bytes(w):
     """Algorithmic bytes of one launch of the dominant kernel: every slot of
-    every macro is read once and written once (the 2D apply writes its
-    interface points in the same launch, the 3D and P2 kernels write the
+    every macro is read once and written once (the P1 applies write their
+    interface points in the same launch, the P2 kernel writes the
     macro-boundary partials)."""
     return w["elem"] * (w["ns"] + (w["ns"] if w["slab"] else w["interior"]))
 
@@ -834,8 +828,8 @@ def main():
                 "traffic": ncu_traffic("%s_%s_%s" % ("k_p2_rows" if v["op"] == "p2" else v["kernel"],
                                                      {H.F64: "f64", H.F32: "f32", H.F64_IEEE: "f64_ieee"}[vcode],
                                                      name))})
-            if v["kernel"] == "k_slab3d":  # the work split the refinement's autotuner picked
-                variants[-1]["slab_z_ranges_per_macro"] = v["M"].autotune_choice(v["L"], vcode)
+            if v["kernel"] == "apply3d":  # the work split the refinement's autotuner picked
+                variants[-1]["z_ranges_per_macro"] = v["M"].autotune_choice(v["L"], vcode)
             if name == WORKLOAD and vcode == H.F64_IEEE:
                 # the native fp64 apply is bound by the fp64 pipe: 7 fp64
                 # operations per macro-interior point (one multiply, three

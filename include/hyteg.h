@@ -109,7 +109,7 @@ int hyteg_mesh_create(int dim, int64_t n_verts, const double* coords, int64_t n_
  * interface tables and the kernels' work lists.  Allocates a few small device
  * tables with cudaMalloc (size O(cells * levels + interface primitives)),
  * owned by the mesh.  Synchronous.  May be called again with a larger level.
- * Levels of at least 2^20 slots are autotuned here: the 3D slab kernel (n <=
+ * Levels of at least 2^20 slots are autotuned here: the 3D kernel (8 < n <=
  * 64) for several work splits (float-float and fp32; native fp64 takes the
  * float-float choice), the 2D kernel for tiles of 8, 16, 32 and 64 rows (each
  * element type), timed on two scratch float64 vectors of the level's size
@@ -122,9 +122,9 @@ int hyteg_mesh_refine(hyteg_mesh* mesh, int max_level);
 
 /* What the autotuner picked on `level` for element type `dtype` (HYTEG_F64,
  * HYTEG_F32, HYTEG_F64_IEEE).  3D: the number of z-ranges every
- * macro-tetrahedron is cut into for the slab kernel, one thread block each;
- * 0 when the level was not autotuned (n > 64, or fewer than 2^20 slots: two
- * z-ranges).  2D: the rows per macro-interior tile (8, 16, 32 or 64), timed
+ * macro-tetrahedron is cut into for the kernel that marches columns through
+ * its slices; 0 when the level was not autotuned (n <= 8, n > 64, or fewer than
+ * 2^20 slots).  2D: the rows per macro-interior tile (8, 16, 32 or 64), timed
  * on levels of at least 2^20 slots; 0 when the level keeps the default
  * tiles (64 rows for float64, 16 for fp32, fewer on levels with few tiles).
  * Errors: HYTEG_EINVAL (null, dtype), HYTEG_ESTATE (level not refined). */

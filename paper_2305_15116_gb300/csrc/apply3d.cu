@@ -1,16 +1,19 @@
-// 3D apply and sweeps of small vectors: one thread per macro-interior point,
-// neighbours straight from memory, and the interface points in the same
-// launch (iface3d.cuh).
+// 3D apply and sweeps (15-point Kuhn stencil): one launch completes the
+// macro-interior and the interface points (iface3d.cuh).  Large vectors march
+// columns through the slices (march3d.cuh); small ones take the direct form
+// below, one thread per macro-interior point, neighbours straight from memory.
 //
 // The 15-point Kuhn stencil in the direct form reads every value 15 times,
 // through L1 and L2; on a level whose vector stays in L2 what counts is the
 // length of the chain of dependent loads, and here it is one table entry
 // (read before the previous kernel has finished) and one round of loads.
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+#include <type_traits>
 #include <vector>
 
-#include "fallback.cuh"
-#include "group.cuh"
-#include "iface3d.cuh"
+#include "march3d.cuh"
 
 namespace hyteg {
 
@@ -82,10 +85,8 @@ struct Direct3 {
     T* y;
     const int2* pts;  // interior points of a macro: (slot, A | M << 16)
     int n_pts, bpm;   // per macro: points, blocks
-    const int4* items;
-    int n_items, n_if_blocks;
-    const Prim* prims;
-    const Inc* incs;
+    int n_if_blocks;
+    Iface3<T> f;
     StencilPtr st;
     ModeArgs md;
     int n;
@@ -93,12 +94,8 @@ struct Direct3 {
   };
   static __device__ __forceinline__ void run(const Prm& p, int block, int) {
     if (block < p.n_if_blocks) {
-      const int item = 2 * block + (int)(threadIdx.x >> 7);
-      if (item >= p.n_items) return;
-      const int4 it = p.items[item];
-      const Prim pr = p.prims[it.x];
-      pdl_wait();
-      iface3d_item<MODE, P::kPoison, T>(p.x, p.y, it, (int)(threadIdx.x & 127), pr, p.incs, p.n, p.S, p.st, p.md);
+      const int u = (kThreads / 32) * block + (int)(threadIdx.x >> 5);
+      if (u < p.f.n_units) iface3d_unit<MODE, P::kPoison, T>(p.x, p.y, p.f, u, p.n, p.S, p.st, p.md);
       return;
     }
     const int b = block - p.n_if_blocks;
@@ -146,6 +143,33 @@ struct Direct3 {
   }
 };
 
+template <class T>
+const T* face_table(const LevelDev& L);
+template <>
+const double* face_table<double>(const LevelDev& L) {
+  return L.wf64;
+}
+template <>
+const float* face_table<float>(const LevelDev& L) {
+  return L.wf32;
+}
+
+template <class T>
+Iface3<T> iface_of(const Mesh& m, const LevelDev& L) {
+  Iface3<T> f;
+  f.items = L.if3;
+  f.n_items = L.n_if3_ev;
+  f.per_face = std::max(1, (L.n_face_pts + 31) / 32);
+  f.n_pts = L.n_face_pts;
+  f.n_faces = L.n_face3;
+  f.n_units = L.n_if3_ev + f.per_face * L.n_face3;
+  f.faces = L.face3;
+  f.ab = L.face_ab;
+  f.incs = m.d_incs;
+  f.wf = face_table<T>(L);
+  return f;
+}
+
 template <class P, int MODE>
 cudaError_t launch_direct(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
                           const ModeArgs* md, int count, cudaStream_t s) {
@@ -164,38 +188,252 @@ cudaError_t launch_direct(const Mesh* const* ms, const int* levels, const void* 
     p.pts = L.pts3;
     p.n_pts = L.n_pts3;
     p.bpm = (L.n_pts3 + B::kThreads - 1) / B::kThreads;
-    p.items = L.if3;
-    p.n_items = L.n_if3;
-    p.n_if_blocks = (L.n_if3 + 1) / 2;
-    p.prims = m.d_prims;
-    p.incs = m.d_incs;
+    p.f = iface_of<T>(m, L);
     p.st = StencilPtr{L.st64, L.st32, L.st_hi, L.st_lo};
     p.md = md ? md[i] : ModeArgs{nullptr, nullptr, 0.0};
     p.n = L.n;
     p.S = L.slots_per_macro;
+    p.n_if_blocks = (p.f.n_units + B::kThreads / 32 - 1) / (B::kThreads / 32);
     prm.push_back(p);
     blocks.push_back(p.n_if_blocks + p.bpm * int(m.n_cells));
   }
   return launch_group<B>(prm.data(), blocks.data(), count, s);
 }
 
+// Work of the columns' march over one macro pair: (first column, z0, z1, -)
+// per block, the longest first; the largest extent of a block's columns with
+// their neighbour rows, in elements.
+struct MarchList {
+  std::vector<int4> work;
+  int stride = 32;
+};
+MarchList march_list(int n, int chunks, bool dense) {
+  MarchList r;
+  auto row = [](int64_t t) {
+    int64_t j = int64_t((std::sqrt(8.0 * double(t) + 1.0) - 1.0) / 2.0);
+    while (j * (j + 1) / 2 > t) --j;
+    while ((j + 1) * (j + 2) / 2 <= t) ++j;
+    return int(j);
+  };
+  std::vector<std::pair<int64_t, int4>> items;
+  for (const int4& z : z_ranges(n, chunks)) {
+    const int zlo = std::max(1, z.y), kmax = n - 1 - zlo;
+    if (kmax < 2 || z.z <= zlo) continue;
+    // columns of rows 2 .. kmax: dense, the interior ones; else all as they lie
+    const int first = dense ? 0 : 3, end = dense ? kmax * (kmax - 1) / 2 : (kmax + 1) * (kmax + 2) / 2;
+    const int all = dense ? (n - 2) * (n - 3) / 2 : 0x7FFFFFFF;
+    for (int t = first; t < end; t += MARCH_COLS) {
+      int k0, k1, q0, q1;
+      if (dense) {
+        const int u = std::min(t + MARCH_COLS, all) - 1;
+        k0 = row(t) + 2, k1 = row(u) + 2;
+        q0 = k0 * (k0 + 1) / 2 + 1 + t - (k0 - 2) * (k0 - 1) / 2;
+        q1 = k1 * (k1 + 1) / 2 + 1 + u - (k1 - 2) * (k1 - 1) / 2;
+      } else {
+        q0 = t, q1 = t + MARCH_COLS - 1;
+        k0 = row(q0), k1 = row(q1);
+      }
+      r.stride = std::max(r.stride, (q1 + k1 + 2) - (q0 - k0 - 1) + 1);
+      const int64_t len = std::min(z.z - 1, n - 1 - k0) - zlo + 3;
+      items.push_back({len, make_int4(t, z.y, z.z, 0)});
+    }
+  }
+  std::stable_sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  for (const auto& i : items) r.work.push_back(i.second);
+  return r;
+}
+
+constexpr size_t kSmemMax = 226 * 1024;  // beside the 128 B of static shared memory
+// macro pairs whose blocks lie together: about so many blocks (a few per
+// SM), so that a column range finds its neighbour rows in L2
+constexpr int kChunkBlocks = 4096;
+// below so many march blocks the interface step takes blocks of its own
+constexpr int kOwnIfaceBlocks = 1024;
+
+template <class P, int MODE, int STRIDE>
+cudaError_t march_attr() {
+  using B = March3<P, MODE, STRIDE>;
+  static_assert(B::smem_bytes() <= kSmemMax, "the ring does not fit");
+  static std::once_flag once;
+  static cudaError_t err = cudaSuccess;
+  std::call_once(once, [] {
+    err = cudaFuncSetAttribute(k_group<B, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::smem_bytes());
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(k_group<B, kGroupMax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)B::smem_bytes());
+  });
+  return err;
+}
+
+template <class P, int MODE, int STRIDE>
+cudaError_t launch_march_s(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
+                           const ModeArgs* md, int count, cudaStream_t s, const March3Work* over) {
+  using B = March3<P, MODE, STRIDE>;
+  using T = typename P::T;
+  constexpr int dt = sizeof(T) == 4 ? 2 : (P::kPoison ? 1 : 3);
+  const cudaError_t attr = march_attr<P, MODE, STRIDE>();
+  if (attr != cudaSuccess) return attr;
+  std::vector<typename B::Prm> prm;
+  std::vector<int> blocks;
+  for (int i = 0; i < count; ++i) {
+    const Mesh& m = *ms[i];
+    const LevelDev& L = m.levels[levels[i]];
+    const March3Work& w = over ? *over : L.march[dt];
+    typename B::Prm p;
+    p.x = static_cast<const T*>(xs[i]);
+    p.y = static_cast<T*>(ys[i]);
+    p.work = w.work;
+    p.n_work = w.n_work;
+    p.n_cells = int(m.n_cells);
+    p.n_pairs = int((m.n_cells + 1) / 2);
+    p.per_chunk = std::max(1, std::min(p.n_pairs, (kChunkBlocks + w.n_work - 1) / std::max(1, w.n_work)));
+    p.f = iface_of<T>(m, L);
+    p.st = StencilPtr{L.st64, L.st32, L.st_hi, L.st_lo};
+    p.md = md ? md[i] : ModeArgs{nullptr, nullptr, 0.0};
+    p.n = L.n;
+    p.S = L.slots_per_macro;
+    if (w.stride > STRIDE) return cudaErrorInvalidValue;
+    p.n_march = int64_t(p.n_work) * p.n_pairs;
+    const int64_t all = p.n_march + (p.n_march < kOwnIfaceBlocks ? (p.f.n_units + 7) / 8 : 0);
+    if (all > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    prm.push_back(p);
+    blocks.push_back(int(all));
+  }
+  return launch_group<B>(prm.data(), blocks.data(), count, s, B::smem_bytes());
+}
+
+// The slot size is a constant of the kernel: the columns of a block with their
+// neighbour rows, 256 + 2n, for n up to 128, 512 and 2048 (float-float up to
+// 512, LevelDev::ff_ok).
+template <class P, int MODE>
+cudaError_t launch_march(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
+                         const ModeArgs* md, int count, cudaStream_t s, const March3Work* over) {
+  const int n = ms[0]->levels[levels[0]].n;
+  if (n <= 128) return launch_march_s<P, MODE, 512>(ms, levels, xs, ys, md, count, s, over);
+  if (n <= 512) return launch_march_s<P, MODE, 1280>(ms, levels, xs, ys, md, count, s, over);
+  if constexpr (!P::kPoison) return launch_march_s<P, MODE, 4352>(ms, levels, xs, ys, md, count, s, over);
+  return cudaErrorInvalidValue;
+}
+
+// The members whose vectors are small take the direct kernel, the others the
+// march; each kind shares its launches.
+template <class P, int MODE>
+cudaError_t launch_t(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
+                     const ModeArgs* md, int count, cudaStream_t s) {
+  // native fp64 is bound by the fp64 pipe either way, and the direct kernel's
+  // occupancy suits it better (level 6, 384 macro-tets: 488 against 600 us)
+  constexpr bool native = std::is_same<P, ArF64Native>::value;
+  auto takes_direct = [](const LevelDev& L) { return L.direct3 || (native && L.pts3); };
+  if (count == 1)
+    return takes_direct(ms[0]->levels[levels[0]]) ? launch_direct<P, MODE>(ms, levels, xs, ys, md, 1, s)
+                                                  : launch_march<P, MODE>(ms, levels, xs, ys, md, 1, s, nullptr);
+  for (int direct = 0; direct < 2; ++direct) {
+    std::vector<const Mesh*> mm;
+    std::vector<int> lv;
+    std::vector<const void*> xx;
+    std::vector<void*> yy;
+    std::vector<ModeArgs> mo;
+    for (int i = 0; i < count; ++i) {
+      if (int(takes_direct(ms[i]->levels[levels[i]])) != direct) continue;
+      mm.push_back(ms[i]);
+      lv.push_back(levels[i]);
+      xx.push_back(xs[i]);
+      yy.push_back(ys[i]);
+      if (md) mo.push_back(md[i]);
+    }
+    if (mm.empty()) continue;
+    const int k = int(mm.size());
+    const ModeArgs* mp = md ? mo.data() : nullptr;
+    const cudaError_t e =
+        direct ? launch_direct<P, MODE>(mm.data(), lv.data(), xx.data(), yy.data(), mp, k, s)
+               : launch_march<P, MODE>(mm.data(), lv.data(), xx.data(), yy.data(), mp, k, s, nullptr);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 template <int MODE>
-cudaError_t launch_direct_dt(int dtype, const Mesh* const* ms, const int* levels, const void* const* xs,
-                             void* const* ys, int count, cudaStream_t s) {
+cudaError_t launch_dt(int dtype, const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
+                      int count, cudaStream_t s) {
   switch (dtype) {
-    case 1: return launch_direct<ArF64FF, MODE>(ms, levels, xs, ys, nullptr, count, s);
-    case 2: return launch_direct<ArF32, MODE>(ms, levels, xs, ys, nullptr, count, s);
-    case 3: return launch_direct<ArF64Native, MODE>(ms, levels, xs, ys, nullptr, count, s);
+    case 1: return launch_t<ArF64FF, MODE>(ms, levels, xs, ys, nullptr, count, s);
+    case 2: return launch_t<ArF32, MODE>(ms, levels, xs, ys, nullptr, count, s);
+    case 3: return launch_t<ArF64Native, MODE>(ms, levels, xs, ys, nullptr, count, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
+// Sum of the copies' partial rows that y holds (Dirichlet points: y = x).
+template <class T>
+struct Sum3 {
+  static constexpr int kThreads = 256;
+  static constexpr bool kLateWait = true;
+  struct Prm {
+    const T* x;
+    T* y;
+    const If3Item* items;
+    int n_items;
+    const Inc* incs;
+    int n;
+    int64_t S;
+  };
+  static __device__ __forceinline__ void run(const Prm& p, int block, int) {
+    const int item = (kThreads / 32) * block + (int)(threadIdx.x >> 5);
+    if (item >= p.n_items) return;
+    const If3Item it = p.items[item];
+    pdl_wait();
+    iface3d_item<MODE_SUM, false, T>(p.x, p.y, it.work, (int)(threadIdx.x & 31), it.prim, p.incs, p.n, p.S, StencilPtr{},
+                                     ModeArgs{});
+  }
+};
+
 }  // namespace
 
-cudaError_t launch_direct3d_group(int dtype, bool partial, const Mesh* const* ms, const int* levels,
-                                  const void* const* xs, void* const* ys, int count, cudaStream_t s) {
-  return partial ? launch_direct_dt<MODE_PARTIAL>(dtype, ms, levels, xs, ys, count, s)
-                 : launch_direct_dt<MODE_APPLY>(dtype, ms, levels, xs, ys, count, s);
+cudaError_t launch_apply3d_group(int dtype, bool partial, const Mesh* const* ms, const int* levels,
+                                 const void* const* xs, void* const* ys, int count, cudaStream_t s) {
+  if (count <= 0) return cudaSuccess;
+  return partial ? launch_dt<MODE_PARTIAL>(dtype, ms, levels, xs, ys, count, s)
+                 : launch_dt<MODE_APPLY>(dtype, ms, levels, xs, ys, count, s);
+}
+
+cudaError_t launch_march3d_work(int dtype, const Mesh& m, int level, const March3Work& work, const void* x, void* y,
+                                cudaStream_t s) {
+  const Mesh* mp = &m;
+  switch (dtype) {
+    case 1: return launch_march<ArF64FF, MODE_APPLY>(&mp, &level, &x, &y, nullptr, 1, s, &work);
+    case 2: return launch_march<ArF32, MODE_APPLY>(&mp, &level, &x, &y, nullptr, 1, s, &work);
+    case 3: return launch_march<ArF64Native, MODE_APPLY>(&mp, &level, &x, &y, nullptr, 1, s, &work);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_sum_copies3d(const Mesh* const* ms, const int* levels, const double* const* xs, double* const* ys,
+                                int count, cudaStream_t s) {
+  using B = Sum3<double>;
+  std::vector<B::Prm> prm;
+  std::vector<int> blocks;
+  for (int i = 0; i < count; ++i) {
+    const LevelDev& L = ms[i]->levels[levels[i]];
+    prm.push_back({xs[i], ys[i], L.if3, L.n_if3, ms[i]->d_incs, L.n, L.slots_per_macro});
+    blocks.push_back((L.n_if3 + B::kThreads / 32 - 1) / (B::kThreads / 32));
+  }
+  return launch_group<B>(prm.data(), blocks.data(), count, s);
+}
+
+cudaError_t apply3d_prepare(int n) {
+  cudaError_t e = cudaSuccess;
+  if (n <= 128) {
+    e = march_attr<ArF64FF, MODE_APPLY, 512>();
+    if (e == cudaSuccess) e = march_attr<ArF32, MODE_APPLY, 512>();
+    if (e == cudaSuccess) e = march_attr<ArF64Native, MODE_APPLY, 512>();
+  }
+  return e;
+}
+
+void march3d_lists(int n, int chunks, int dtype, std::vector<int4>& work, int& stride) {
+  MarchList l = march_list(n, chunks, dtype == 1);
+  work = std::move(l.work);
+  stride = l.stride;
 }
 
 }  // namespace hyteg

@@ -1,4 +1,4 @@
-// Autotuners run at refinement: the 3D slab kernel's work split (z-ranges
+// Autotuners run at refinement: the 3D march's work split (z-ranges
 // per macro-tet) and the 2D kernel's tile height.
 #include <array>
 #include <map>
@@ -9,20 +9,20 @@
 
 namespace hyteg {
 
-// ---- autotuner of the slab work split -------------------------------------------
-// How many z-ranges a macro is cut into trades the waves of CTAs over the SMs
-// (which depend on the blocks per SM of each element type) against the
-// per-item cost of loading the first three slices.  On first use of a level
-// size the kernel is timed for each candidate on scratch vectors (the best
-// of two launches each, so that a concurrent workload inflates no candidate
-// in particular) and the fastest list is kept; the choice is cached per
-// (macro count, level, element type) for the process.  Float-float and fp32
-// are timed; native fp64, which fits the same blocks per SM as float-float,
-// takes float-float's choice.  Levels below 2^20 slots keep two z-ranges:
-// their kernels take a few microseconds, and a solve server meets many such
-// sizes once each.
-cudaError_t slab3d_autotune(Mesh& m, LevelDev& L) {
-  if (L.n_slabs == 0 || m.autotune == 0) return cudaSuccess;
+// ---- autotuner of the 3D march's work split ---------------------------------------
+// How many z-ranges a macro is cut into trades the balance of the blocks over
+// the SMs (a block's time is its number of slices) against the two slices per
+// range that are read beside the written ones.  On first use of a level size
+// the kernel is timed for each candidate on scratch vectors (the best of two
+// launches each, so that a concurrent workload inflates no candidate in
+// particular) and the fastest list is kept; the choice is cached per (macro
+// count, level, element type) for the process.  Float-float and fp32 are
+// timed; native fp64, which the direct kernel takes, reports float-float's
+// choice.  Levels below 2^20 slots take the direct kernel; above n = 64, n/32
+// ranges.
+cudaError_t march3d_autotune(Mesh& m, int level) {
+  LevelDev& L = m.levels[level];
+  if (L.direct3 || L.n > 64 || m.autotune == 0) return cudaSuccess;
   const int64_t total = L.slots_per_macro * m.n_cells;
   if (total < (int64_t(1) << 20)) return cudaSuccess;
   static std::mutex mu;
@@ -45,7 +45,7 @@ cudaError_t slab3d_autotune(Mesh& m, LevelDev& L) {
   };
   for (int dt = 1; dt <= 3 && err == cudaSuccess; ++dt) {
     const std::array<int64_t, 3> key{m.n_cells, L.n, dt == 3 ? 1 : dt};
-    int best = dt == 3 ? L.slab_chunks[1] : 0;
+    int best = dt == 3 ? L.z_chunks[1] : 0;
     if (best == 0) {
       std::lock_guard<std::mutex> lk(mu);
       auto it = cache.find(key);
@@ -75,16 +75,13 @@ cudaError_t slab3d_autotune(Mesh& m, LevelDev& L) {
       }
       float best_ms = 0.0f;
       for (int c : kCand) {
-        const std::vector<int4> items = slab_work_list(L.n, m.n_cells, c);
-        int4* d_items = nullptr;
-        if ((err = dev_alloc(m, (void**)&d_items, items.size() * sizeof(int4))) != cudaSuccess) break;
-        err = dev_upload(m, d_items, items.data(), items.size() * sizeof(int4));
-        if (err == cudaSuccess) err = dev_sync(m);
+        if ((err = set_march(m, L, dt, c)) != cudaSuccess) break;
+        if ((err = dev_sync(m)) != cudaSuccess) break;
         float ms = 0.0f;
         const int first = c == kCand[0] ? 0 : 1;  // one warm-up launch per element type
         for (int rep = first; rep < 3 && err == cudaSuccess; ++rep) {
           if ((err = cudaEventRecord(e0, s)) != cudaSuccess) break;
-          if ((err = launch_slab3d_items(dt, L, d_items, int(items.size()), x, y, s)) != cudaSuccess) break;
+          if ((err = launch_march3d_work(dt, m, level, L.march[dt], x, y, s)) != cudaSuccess) break;
           if ((err = cudaEventRecord(e1, s)) != cudaSuccess) break;
           if ((err = cudaEventSynchronize(e1)) != cudaSuccess) break;
           float t = 0.0f;
@@ -92,7 +89,6 @@ cudaError_t slab3d_autotune(Mesh& m, LevelDev& L) {
           if (rep == 1 || (rep > 1 && t < ms)) ms = t;
         }
         const cudaError_t ef = cudaStreamSynchronize(s);
-        dev_free(m, d_items);
         if (err == cudaSuccess) err = ef;
         if (err != cudaSuccess) break;
         if (best == 0 || ms < best_ms) {
@@ -104,13 +100,8 @@ cudaError_t slab3d_autotune(Mesh& m, LevelDev& L) {
       std::lock_guard<std::mutex> lk(mu);
       cache[key] = best;
     }
-    if (best != 2) {  // the default list holds two z-ranges per macro
-      const std::vector<int4> items = slab_work_list(L.n, m.n_cells, best);
-      if ((err = dev_alloc(m, (void**)&L.slabs_dt[dt], items.size() * sizeof(int4))) != cudaSuccess) break;
-      if ((err = dev_upload(m, L.slabs_dt[dt], items.data(), items.size() * sizeof(int4))) != cudaSuccess) break;
-      L.n_slabs_dt[dt] = int(items.size());
-    }
-    L.slab_chunks[dt] = best;
+    if ((err = set_march(m, L, dt, best)) != cudaSuccess) break;
+    L.z_chunks[dt] = best;
   }
   if (err == cudaSuccess) err = dev_sync(m);
   cleanup();

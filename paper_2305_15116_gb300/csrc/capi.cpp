@@ -112,9 +112,9 @@ int hyteg_mesh_refine(hyteg_mesh* mesh, int max_level) {
       }
       m.levels.push_back(L);
       m.max_level = l;
-      if (m.dim == 3) {  // pick the 3D slab kernel's work split for this level
-        e = hyteg::slab3d_autotune(m, m.levels.back());
-        if (e != cudaSuccess) return cuda_fail(e, "slab work-split autotuning");
+      if (m.dim == 3) {  // pick the 3D march's work split for this level
+        e = hyteg::march3d_autotune(m, l);
+        if (e != cudaSuccess) return cuda_fail(e, "3D work-split autotuning");
       } else {  // and the 2D kernel's tile height
         e = hyteg::tiles2d_autotune(m, m.levels.back());
         if (e != cudaSuccess) return cuda_fail(e, "2D tile autotuning");
@@ -156,7 +156,7 @@ int hyteg_autotune_choice(const hyteg_mesh* mesh, int level, int dtype, int* val
   if (!value) return fail(HYTEG_EINVAL, "value is NULL");
   if (dtype != HYTEG_F64 && dtype != HYTEG_F32 && dtype != HYTEG_F64_IEEE) return fail(HYTEG_EINVAL, "bad dtype");
   const hyteg::LevelDev& L = mesh->m.levels[level];
-  *value = mesh->m.dim == 3 ? L.slab_chunks[dtype] : L.tile_rows[dtype];
+  *value = mesh->m.dim == 3 ? L.z_chunks[dtype] : L.tile_rows[dtype];
   return HYTEG_OK;
 }
 
@@ -513,16 +513,6 @@ int hyteg_solve_two_part_group(hyteg_mesh* const* meshes, int count, int level, 
       if (ms[j] == ms[i]) return fail(HYTEG_EINVAL, "a mesh appears twice" + at);
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // 3D levels above the slab kernel's (n > 64) have no group launch: the
-  // meshes are solved one after another
-  if (ms[0]->dim == 3 && ms[0]->levels[level].n_slabs == 0) {
-    for (int i = 0; i < count; ++i) {
-      const cudaError_t e = hyteg::mg_solve(*ms[i], level, mode, b[i], u[i], u_lo[i], rtol, max_iter, s, iters + i,
-                                            relres + i);
-      if (e != cudaSuccess) return cuda_fail(e, "solve");
-    }
-    return HYTEG_OK;
-  }
   const cudaError_t e = hyteg::mg_solve_group(ms.data(), count, level, mode, b, u, u_lo, rtol, max_iter, s, iters,
                                               relres);
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, "group solve");

@@ -52,6 +52,12 @@ struct late_wait : std::false_type {};
 template <class B>
 struct late_wait<B, std::void_t<decltype(B::kLateWait)>> : std::bool_constant<B::kLateWait> {};
 
+// A body built for a number of blocks per SM declares kMinBlocks.
+template <class B, class = void>
+struct min_blocks : std::integral_constant<int, 0> {};
+template <class B>
+struct min_blocks<B, std::void_t<decltype(B::kMinBlocks)>> : std::integral_constant<int, B::kMinBlocks> {};
+
 constexpr int kGroupMax = 16;  // meshes per group launch
 
 template <class Prm, int N>
@@ -75,7 +81,7 @@ __device__ __forceinline__ int group_entry(const GroupArgs<Prm, N>& g, int block
 }
 
 template <class Body, int N>
-__global__ void __launch_bounds__(Body::kThreads) k_group(const __grid_constant__ GroupArgs<typename Body::Prm, N> g) {
+__global__ void __launch_bounds__(Body::kThreads, min_blocks<Body>::value) k_group(const __grid_constant__ GroupArgs<typename Body::Prm, N> g) {
   pdl_trigger();
   if constexpr (!late_wait<Body>::value) pdl_wait();
   const int e = N == 1 ? 0 : group_entry(g, (int)blockIdx.x);

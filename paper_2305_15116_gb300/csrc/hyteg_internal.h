@@ -27,6 +27,37 @@ constexpr int C3 = 0;      // index of the centre weight in 3D
 
 struct Off3 { int dx, dy, dz; };
 
+// Interface primitive (coarse vertex, edge or face).
+struct Prim {
+  int type;        // 0 vertex, 1 edge, 2 face
+  int boundary;    // 1 if all its refined points are Dirichlet DoFs
+  int inc_begin;   // first entry in the incidence table
+  int inc_count;   // number of incident cells (ascending cell id)
+};
+
+// Item of the 3D interface work list: (-, first point, points, lanes per
+// point) of one primitive.
+struct If3Item {
+  int4 work;
+  Prim prim;
+};
+
+// Work of the 3D column march over one macro pair (march3d.cuh).
+struct March3Work {
+  int4* work = nullptr;
+  int n_work = 0;
+  int stride = 0;  // elements per slice and macro in shared memory
+};
+
+// A coarse face: its copies' cells (second -1: none) and per copy the local
+// coordinates as affine functions of a face point's canonical weights (a, b):
+// for every axis two bits each for the coefficients of 1 (0 or n), a and b (0,
+// 1, or 3 for -1), and the corner that the face does not hold (bits 18, 19).
+struct Face3Rec {
+  int cell0, cell1;
+  unsigned map0, map1;
+  int dirichlet, pad[3];
+};
 // Device tables of one refinement level.
 struct LevelDev {
   int level = -1;
@@ -53,41 +84,28 @@ struct LevelDev {
   // interface work list: int4 (prim, b, a0, a1)
   int4* items = nullptr;
   int n_items = 0;
-  // 3D: slots of every copy of every interface point (work-list order) and
-  // each item's first entry
-  int64_t* if_slots = nullptr;
-  int64_t* if_item_base = nullptr;
-  int64_t n_if_slots = 0;
-  // points with two copies (inside the domain) or one (Dirichlet), reduced
-  // by a flat kernel: (slot, slot) or (slot, -2); each item's first entry
-  // (-1: the item's points are not in the table); the items left to the
-  // general reduction
-  longlong2* if_pairs = nullptr;
-  int64_t n_if_pairs = 0;
-  int64_t* if_flat_base = nullptr;
-  int* if_rest = nullptr;
-  int n_if_rest = 0;
   // 3D: interface work list of the one-launch apply, int4 (prim, first
   // point, points, lanes per point)
-  int4* if3 = nullptr;
-  int n_if3 = 0;
-  // 3D, small vectors: one thread per macro-interior point, from the table of
-  // the macro's interior points (slot, row length | slice side << 16)
+  // first the edges and vertices (n_if3_ev items), then the faces, which the
+  // apply takes from face3 instead
+  If3Item* if3 = nullptr;
+  int n_if3 = 0, n_if3_ev = 0;
+  Face3Rec* face3 = nullptr;
+  int n_face3 = 0, n_face_pts = 0;
+  unsigned* face_ab = nullptr;  // interior points of a face, a | b << 16
+  double* wf64 = nullptr;    // [cell][opposite corner][12]: the 11 weights of a face point's partial row
+  float* wf32 = nullptr;
+  // 3D, small vectors (direct3) and native fp64: one thread per macro-interior
+  // point, from the table of the macro's interior points (slot, row length |
+  // slice side << 16)
   bool direct3 = false;
   int2* pts3 = nullptr;
   int n_pts3 = 0;
-  // 3D row-kernel work list: int4 (x0, y0, y1, z): lattice columns x0-1..x0+30
-  // (x0..x0+29 written), rows y0..y1-1 of slice z of one macro
-  int4* r3_tiles = nullptr;
-  int n_r3_tiles = 0;
-  // 3D slab work list (levels with n <= 64): int4 (macro, z0, z1, 0)
-  int4* slabs = nullptr;
-  int n_slabs = 0;
-  // per element type (1 float-float, 2 fp32, 3 native fp64): the slab work
-  // list the autotuner picked (nullptr: `slabs`), and its z-ranges per macro
-  int4* slabs_dt[4] = {nullptr, nullptr, nullptr, nullptr};
-  int n_slabs_dt[4] = {0, 0, 0, 0};
-  int slab_chunks[4] = {0, 0, 0, 0};
+  // 3D, large vectors, per element type (1 float-float, 2 fp32, 3 native
+  // fp64): the columns' march, and the z-ranges per macro that the autotuner
+  // picked for it (0: not tuned, two ranges)
+  March3Work march[4];
+  int z_chunks[4] = {0, 0, 0, 0};
   // host copy of the class stencils (multigrid set-up)
   std::vector<double> st_host;
   // P2 (2D): class stencils [cell][P2W] and the edge interface work list
@@ -120,7 +138,6 @@ int64_t p2_edge_slots(int level);  // n(n+1)/2 edges of one group per macro
 bool ff_weights_in_range(const std::vector<double>& st, int per_stencil);
 int64_t p2_slots_per_macro(int level);
 
-// Interface primitive (coarse vertex, edge or face) and its incident cells.
 #ifdef __CUDACC__
 // Macro index of a slot index i (slots per macro S >= 2) without a 64-bit
 // division per element: for i, S < 2^32 the quotient is the high 64 bits of
@@ -137,12 +154,6 @@ struct SlotDiv {
 };
 #endif
 
-struct Prim {
-  int type;        // 0 vertex, 1 edge, 2 face
-  int boundary;    // 1 if all its refined points are Dirichlet DoFs
-  int inc_begin;   // first entry in the incidence table
-  int inc_count;   // number of incident cells (ascending cell id)
-};
 
 // One incidence: the cell and the local corner index (0..dim) of each of the
 // primitive's canonical vertices in that cell (-1 if unused).
@@ -232,7 +243,7 @@ struct Mesh {
   Solver* solver = nullptr;
   ProblemDev problem;
   DevMem mem;
-  // slab work-split autotuning at refinement: 2 time the candidates on a
+  // work-split autotuning at refinement: 2 time the candidates on a
   // cache miss, 1 only take cached choices (meshes built by the solve server,
   // whose timings would run among other requests' kernels), 0 off
   int autotune = 2;
@@ -245,13 +256,16 @@ void set_last_error(const std::string& msg);
 // Returns an error message, empty on success.
 std::string build_topology(Mesh& m);
 std::string build_level(Mesh& m, int level, LevelDev& out);
-// 3D slab work items (macro, z0, z1): every macro cut into `chunks` z-ranges
-// of about equal point counts
-std::vector<int4> slab_work_list(int n, int64_t n_cells, int chunks);
-// Time the slab kernel on this level for several z-range counts per element
+// z-ranges (-, z0, z1, -): a macro cut into `chunks` ranges of about equal
+// point counts
+std::vector<int4> z_ranges(int n, int chunks);
+// the work list of the 3D march for `chunks` z-ranges, built and uploaded
+void march3d_lists(int n, int chunks, int dtype, std::vector<int4>& work, int& stride);
+cudaError_t set_march(const Mesh& m, LevelDev& L, int dt, int chunks);
+// Time the 3D march on this level for several z-range counts per element
 // type and keep the fastest list (levels of at least 2^20 slots; results are
 // cached per (macro count, level size) for the process).  Synchronous.
-cudaError_t slab3d_autotune(Mesh& m, LevelDev& L);
+cudaError_t march3d_autotune(Mesh& m, int level);
 // The 2D macro-interior tiles of one macro (same list for every macro):
 // strips of 62 columns from x = 1, rows cut into chunks of `rows`, ordered
 // row chunk by row chunk.
@@ -340,34 +354,27 @@ cudaError_t launch_sweep2d(int dtype, bool jacobi, const Mesh& m, const LevelDev
 cudaError_t launch_sweep2d_group(bool jacobi, const Mesh* const* ms, const int* levels, const void* const* u,
                                  const void* const* b, const void* const* dinv, const double* omega,
                                  void* const* out, int count, cudaStream_t s);
-// the slab kernel of several 3D meshes (levels with n <= 64) in one launch
-cudaError_t launch_slab3d_group(int dtype, const Mesh* const* ms, const int* levels, const void* const* xs,
-                                void* const* ys, int count, cudaStream_t s);
-cudaError_t launch_slab3d(int dtype, const LevelDev& L, const void* x, void* y, cudaStream_t s);
-// raises the slab kernels' shared-memory limit (once per process; before any
-// stream capture)
-cudaError_t slab3d_prepare();
-// the slab kernel over an explicit work list (the autotuner's candidates)
-cudaError_t launch_slab3d_items(int dtype, const LevelDev& L, const int4* items, int n_items, const void* x,
-                                void* y, cudaStream_t s);
-// Levels whose vectors the direct 3D kernel takes (LevelDev::direct3): up to
-// 2^21 slots it is faster than the slab kernel and its interface launch in
-// every element type (us per apply, direct / slab + interface; float64, fp32,
-// native: 35k slots 11.0 / 21.2, 10.9 / 13.3; 0.47M slots 11.1 / 48.1,
-// 10.9 / 28.7, 14.0 / 78.7; 1.9M slots 37.8 / 62.5, 14.5 / 31.1, 52.6 / 102;
-// at 18M slots 337 / 298, 144 / 131).
+// Levels whose vectors the direct 3D kernel takes (LevelDev::direct3), and the
+// levels with its point table (which native fp64 always uses).
 constexpr int kDirect3MaxN = 64;
-constexpr int64_t kDirect3MaxSlots = int64_t(1) << 21;
-// the direct 3D kernel of several meshes in one launch, interface step
+constexpr int64_t kDirect3MaxSlots = int64_t(1) << 20;
+constexpr int kDirect3TableN = 128;
+// the 3D apply of several meshes, one launch per kernel kind, interface step
 // included (partial: every interface copy keeps its own macro's partial row)
-cudaError_t launch_direct3d_group(int dtype, bool partial, const Mesh* const* ms, const int* levels,
-                                  const void* const* xs, void* const* ys, int count, cudaStream_t s);
-cudaError_t launch_row3d(int dtype, const LevelDev& L, int64_t n_cells, const void* x, void* y, cudaStream_t s);
-cudaError_t build_iface_slots(const Mesh& m, const LevelDev& L, cudaStream_t s);
-cudaError_t launch_interface_reduce(int dtype, const Mesh& m, int level, const void* x, void* y, cudaStream_t s);
-// the interface reduction of several meshes of one dimension
-cudaError_t launch_interface_reduce_group(int dtype, const Mesh* const* ms, const int* levels, const void* const* x,
-                                          void* const* y, int count, cudaStream_t s);
+cudaError_t launch_apply3d_group(int dtype, bool partial, const Mesh* const* ms, const int* levels,
+                                 const void* const* xs, void* const* ys, int count, cudaStream_t s);
+// the march over an explicit work list (the autotuner's candidates)
+cudaError_t launch_march3d_work(int dtype, const Mesh& m, int level, const March3Work& work, const void* x, void* y,
+                                cudaStream_t s);
+// raises the march kernels' shared-memory limit (once per process; before any
+// stream capture)
+cudaError_t apply3d_prepare(int n);
+// ys hold every copy's partial row: the sums over the copies (Dirichlet: x)
+cudaError_t launch_sum_copies3d(const Mesh* const* ms, const int* levels, const double* const* xs, double* const* ys,
+                                int count, cudaStream_t s);
+// the same in one call for either dimension
+cudaError_t launch_sum_copies(const Mesh* const* ms, const int* levels, const double* const* x, double* const* y,
+                              int count, cudaStream_t s);
 
 // The launch sequence of one apply y = A x (two kernels); `ev_mid`, when not
 // null, is recorded between them.  Returns the failing step in *what.

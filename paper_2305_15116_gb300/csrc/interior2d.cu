@@ -28,7 +28,6 @@
 #include "fallback.cuh"
 #include "group.cuh"
 #include "hyteg_internal.h"
-#include "modes.cuh"
 
 namespace hyteg {
 
@@ -87,6 +86,39 @@ __device__ __forceinline__ bool pair_aligned(const float* p) { return (reinterpr
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// What a launch writes at a point with (A u) = au:
+//   MODE_APPLY:    y = A u
+//   MODE_JACOBI:   y = u + omega dinv (b - A u)   (one weighted Jacobi sweep)
+//   MODE_RESIDUAL: y = b - A u
+// (u = x at the point; b and dinv in the slot layout, copies equal).
+//   MODE_PARTIAL:  y = A u inside the macros; at interface points every copy
+//                  receives its own macro's partial row instead of the sum
+constexpr int MODE_APPLY = 0, MODE_JACOBI = 1, MODE_RESIDUAL = 2, MODE_PARTIAL = 3;
+
+struct ModeArgs {
+  const void* b;
+  const void* dinv;
+  double omega;
+};
+
+// sweep modes inside the macro: u, b and dinv of the point come from the
+// staged rows
+template <int MODE, class T>
+__device__ __forceinline__ T mode_out_staged(T au, T u, T b, T d, double omega) {
+  if (MODE == MODE_APPLY) return au;
+  if (MODE == MODE_RESIDUAL) return b - au;
+  return u + (T)omega * d * (b - au);
+}
+
+template <int MODE, class T>
+__device__ __forceinline__ T mode_out(T au, const T* __restrict__ x, const ModeArgs& md, int64_t i) {
+  if (MODE == MODE_APPLY) return au;
+  const T bi = __ldg(static_cast<const T*>(md.b) + i);
+  if (MODE == MODE_RESIDUAL) return bi - au;
+  const T ui = __ldg(x + i), di = __ldg(static_cast<const T*>(md.dinv) + i);
+  return ui + (T)md.omega * di * (bi - au);
+}
 
 // ---- interface points (coarse vertices and edges), stencil mode ------------
 // Each macro holding a copy contributes its partial row (the class stencil of

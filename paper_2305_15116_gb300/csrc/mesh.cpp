@@ -290,23 +290,30 @@ std::string build_topology(Mesh& m) {
   return "";
 }
 
-std::vector<int4> slab_work_list(int n, int64_t n_cells, int chunks) {
-  // cuts at z where the cumulative slice point count passes c/chunks of the
-  // macro's slots; items ordered by z-range, then macro
-  const int64_t S = (int64_t(n) + 1) * (n + 2) * (n + 3) / 6;
-  std::vector<int> cuts = {0};
-  int64_t acc = 0;
-  for (int z = 0; z <= n; ++z) {
-    const int64_t M = n + 1 - z;
-    acc += M * (M + 1) / 2;
-    if (int(cuts.size()) < chunks && acc * chunks >= S * int64_t(cuts.size()) && z < n) cuts.push_back(z + 1);
+std::vector<int4> z_ranges(int n, int chunks) {
+  std::vector<int4> r;
+  for (int c = 0; c < chunks; ++c) {
+    const int z0 = int(int64_t(n + 1) * c / chunks), z1 = int(int64_t(n + 1) * (c + 1) / chunks);
+    if (z0 < z1) r.push_back(make_int4(0, z0, z1, 0));
   }
-  cuts.push_back(n + 1);
-  std::vector<int4> items;
-  for (size_t c = 0; c + 1 < cuts.size(); ++c)
-    for (int64_t mm = 0; mm < n_cells; ++mm)
-      if (cuts[c] < cuts[c + 1]) items.push_back(make_int4(int(mm), cuts[c], cuts[c + 1], 0));
-  return items;
+  return r;
+}
+
+cudaError_t set_march(const Mesh& m, LevelDev& L, int dt, int chunks) {
+  std::vector<int4> w;
+  March3Work& k = L.march[dt];
+  march3d_lists(L.n, chunks, dt, w, k.stride);
+  dev_free(m, k.work);
+  k.work = nullptr;
+  k.n_work = int(w.size());
+  if (w.empty()) return cudaSuccess;
+  const cudaError_t e = dev_alloc(m, (void**)&k.work, w.size() * sizeof(int4));
+  if (e != cudaSuccess) {
+    k.work = nullptr;
+    k.n_work = 0;
+    return e;
+  }
+  return dev_upload(m, k.work, w.data(), w.size() * sizeof(int4));
 }
 
 void free_level(const Mesh& m, LevelDev& L) {
@@ -318,16 +325,13 @@ void free_level(const Mesh& m, LevelDev& L) {
   dev_free(m, L.tiles32);
   for (int t = 0; t < 4; ++t) dev_free(m, L.tiles_dt[t]);
   dev_free(m, L.items);
-  dev_free(m, L.slabs);
-  for (int t = 0; t < 4; ++t) dev_free(m, L.slabs_dt[t]);
-  dev_free(m, L.r3_tiles);
+  for (int t = 0; t < 4; ++t) dev_free(m, L.march[t].work);
   dev_free(m, L.pts3);
   dev_free(m, L.if3);
-  dev_free(m, L.if_slots);
-  dev_free(m, L.if_item_base);
-  dev_free(m, L.if_pairs);
-  dev_free(m, L.if_flat_base);
-  dev_free(m, L.if_rest);
+  dev_free(m, L.face3);
+  dev_free(m, L.face_ab);
+  dev_free(m, L.wf64);
+  dev_free(m, L.wf32);
   dev_free(m, L.p2_st64);
   dev_free(m, L.p2_st32);
   dev_free(m, L.p2_hi);
@@ -463,7 +467,9 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     sth[i] = float(ws);
     stl[i] = float(ws - double(sth[i]));
   }
-  L.ff_ok = ff_weights_in_range(st, ncls * nw);
+  // a slice's columns with their neighbour rows, split for the 3D march, fit
+  // in shared memory up to n = 512; above, native fp64
+  L.ff_ok = ff_weights_in_range(st, ncls * nw) && (d == 2 || n <= 512);
 
   // ---- 2D macro-interior work lists: strips of columns x chunks of rows ----
   // a warp loads 64 consecutive columns and writes the 62 inner ones.  A warp
@@ -514,13 +520,6 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
   }
   L.n_items = int(items.size());
 
-  // ---- 3D slab work list: every macro cut into two z-ranges of about equal
-  // point counts (n <= 64, where three slices fit in shared memory); the
-  // autotuner may replace it per element type after refinement -------------
-  std::vector<int4> slabs;
-  if (d == 3 && n <= 64) slabs = slab_work_list(n, m.n_cells, 2);
-  L.n_slabs = int(slabs.size());
-
   std::string err;
   if (!(err = upload(m, &L.st64, st)).empty()) return err;
   if (!(err = upload(m, &L.st32, st32)).empty()) return err;
@@ -529,78 +528,70 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
   if (!(err = upload(m, &L.tiles, tiles)).empty()) return err;
   if (!(err = upload(m, &L.tiles32, tiles32)).empty()) return err;
   if (!(err = upload(m, &L.items, items)).empty()) return err;
-  if (!(err = upload(m, &L.slabs, slabs)).empty()) return err;
-  if (d == 3 && !items.empty()) {
-    // the slot table of the interface reduction (built on the device)
-    std::vector<int64_t> base(items.size() + 1, 0);
-    for (size_t i = 0; i < items.size(); ++i)
-      base[i + 1] = base[i] + int64_t(items[i].w - items[i].z) * m.prims[items[i].x].inc_count;
-    L.n_if_slots = base.back();
-    if (!(err = upload(m, &L.if_item_base, base)).empty()) return err;
-    std::vector<int64_t> fbase(items.size(), -1);
-    std::vector<int> rest;
-    int64_t nflat = 0;
-    for (size_t i = 0; i < items.size(); ++i) {
-      const Prim& pr = m.prims[items[i].x];
-      if ((!pr.boundary && pr.inc_count == 2) || (pr.boundary && pr.inc_count == 1)) {
-        fbase[i] = nflat;
-        nflat += items[i].w - items[i].z;
-      } else if (pr.boundary || pr.inc_count > 1) {
-        rest.push_back(int(i));
-      }
-    }
-    L.n_if_pairs = nflat;
-    L.n_if_rest = int(rest.size());
-    if (!(err = upload(m, &L.if_flat_base, fbase)).empty()) return err;
-    if (!(err = upload(m, &L.if_rest, rest)).empty()) return err;
-    if (nflat > 0) {
-      const cudaError_t ep = dev_alloc(m, (void**)&L.if_pairs, size_t(nflat) * sizeof(longlong2));
-      if (ep != cudaSuccess) {
-        L.if_pairs = nullptr;
-        return "device allocation: interface pair table";
-      }
-    }
-    const cudaError_t e = dev_alloc(m, (void**)&L.if_slots, size_t(L.n_if_slots) * sizeof(int64_t));
-    if (e != cudaSuccess) {
-      L.if_slots = nullptr;
-      return "device allocation: interface slot table";
-    }
-    const cudaError_t e2 = build_iface_slots(m, L, m.mem.stream);
-    if (e2 != cudaSuccess) return std::string("cuda: ") + cudaGetErrorString(e2);
-  }
-  if (d == 3) {
-    // row-kernel tiles: every slice z, strips of 30 columns, chunks of 32 rows
-    // (level 7, 384 macro-tets: 3.94 -> 3.50 ms float-float and 1.16 -> 1.11
-    // ms fp32 against 64-row chunks; a warp walks its rows serially)
-    constexpr int R3TH = 32;
-    std::vector<int4> r3;
-    for (int z = 0; z <= n; ++z) {
-      const int M = n + 1 - z;
-      for (int x0 = 0; x0 <= M - 1; x0 += 30)
-        for (int y0 = 0; y0 <= M - 1 - x0; y0 += R3TH)
-          r3.push_back(make_int4(x0, y0, std::min(y0 + R3TH, M - x0), z));
-    }
-    L.n_r3_tiles = int(r3.size());
-    if (!(err = upload(m, &L.r3_tiles, r3)).empty()) return err;
-  }
   if (d == 3) {
     // interface work list of the 3D apply (iface3d.cuh): (prim, first point,
-    // points, lanes per point), at most 128 threads per item
-    std::vector<int4> if3;
+    // points, lanes per point), one warp per item
+    std::vector<If3Item> if3;
     for (size_t p = 0; p < m.prims.size(); ++p) {
       const Prim& pr = m.prims[p];
       const int64_t np = pr.type == 0 ? 1 : pr.type == 1 ? n - 1 : int64_t(n - 1) * (n - 2) / 2;
       int lanes = 1;
       if (pr.inc_count > 2 && pr.inc_count <= 32 && !pr.boundary)
         while (lanes < pr.inc_count) lanes *= 2;
-      const int per = 128 / lanes;
+      const int per = 32 / lanes;
       for (int64_t t = 0; t < np; t += per)
-        if3.push_back(make_int4(int(p), int(t), int(std::min<int64_t>(per, np - t)), lanes));
+        if3.push_back({make_int4(int(p), int(t), int(std::min<int64_t>(per, np - t)), lanes), pr});
     }
     L.n_if3 = int(if3.size());
+    L.n_if3_ev = int(std::count_if(if3.begin(), if3.end(), [](const If3Item& i) { return i.prim.type < 2; }));
+    std::vector<unsigned> ab;
+    for (int b = 1; b <= n - 2; ++b)
+      for (int a = 1; a <= n - 1 - b; ++a) ab.push_back(unsigned(a) | unsigned(b) << 16);
+    auto face_map = [&](const Inc& inc) {
+      // corner c >= 1 is the unit point of axis c-1; weights (n-a-b, a, b)
+      unsigned map = 0;
+      int missing = 6;
+      for (int j = 0; j < 3; ++j) {
+        const int c = inc.corner[j];
+        missing -= c;
+        if (c < 1) continue;
+        const unsigned co = j == 0 ? (1u | 3u << 2 | 3u << 4) : j == 1 ? 1u << 2 : 1u << 4;
+        map |= co << (6 * (c - 1));
+      }
+      return map | unsigned(missing) << 18;
+    };
+    std::vector<Face3Rec> faces;
+    for (const Prim& pr : m.prims) {
+      if (pr.type != 2) continue;
+      const Inc& i0 = m.incs[pr.inc_begin];
+      const Inc& i1 = m.incs[pr.inc_begin + (pr.inc_count > 1 ? 1 : 0)];
+      faces.push_back({i0.cell, pr.inc_count > 1 ? i1.cell : -1, face_map(i0), face_map(i1), pr.boundary, {0, 0, 0}});
+    }
+    // in the order in which the macros are swept, when both copies' macros
+    // are in L2
+    std::stable_sort(faces.begin(), faces.end(), [](const Face3Rec& p, const Face3Rec& q) {
+      return std::max(p.cell0, p.cell1) < std::max(q.cell0, q.cell1);
+    });
+    L.n_face3 = ab.empty() ? 0 : int(faces.size());
+    L.n_face_pts = int(ab.size());
+    if (!(err = upload(m, &L.face3, faces)).empty()) return err;
+    if (!(err = upload(m, &L.face_ab, ab)).empty()) return err;
     if (!(err = upload(m, &L.if3, if3)).empty()) return err;
-    L.direct3 = n <= kDirect3MaxN && L.slots_per_macro * m.n_cells <= kDirect3MaxSlots;
-    if (L.direct3) {  // the macro-interior points in slot order: (slot, A | M << 16)
+    // the face without corner f is x+y+z = n (f = 0) or x, y, z = 0
+    std::vector<double> wf(size_t(m.n_cells) * 4 * 12, 0.0);
+    for (int64_t c = 0; c < m.n_cells; ++c)
+      for (int f = 0; f < 4; ++f) {
+        const int cls = f == 0 ? 8 : 1 << (f - 1);
+        int t = 0;
+        for (int k = 0; k < NW3; ++k)
+          if (inside3(cls, OFF3[k][0], OFF3[k][1], OFF3[k][2]))
+            wf[(size_t(c) * 4 + f) * 12 + t++] = st[(size_t(c) * ncls + cls) * nw + k];
+      }
+    std::vector<float> wf_f(wf.begin(), wf.end());
+    if (!(err = upload(m, &L.wf64, wf)).empty()) return err;
+    if (!(err = upload(m, &L.wf32, wf_f)).empty()) return err;
+    L.direct3 = n <= 8 || (n <= kDirect3MaxN && L.slots_per_macro * m.n_cells <= kDirect3MaxSlots);
+    if (n <= kDirect3TableN) {  // the macro-interior points in slot order: (slot, A | M << 16)
       std::vector<int2> pts;
       int slot = 0;
       for (int z = 0; z <= n; ++z)
@@ -612,6 +603,15 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
             }
       L.n_pts3 = int(pts.size());
       if (!(err = upload(m, &L.pts3, pts)).empty()) return err;
+    }
+    if (!L.direct3) {  // the columns' march (the autotuner may change the z-ranges)
+      const cudaError_t ep = apply3d_prepare(n);
+      if (ep != cudaSuccess) return std::string("cuda: ") + cudaGetErrorString(ep);
+      for (int dt = 1; dt <= 3; ++dt)
+        if (set_march(m, L, dt, std::max(2, n / 32)) != cudaSuccess) {
+          cudaGetLastError();
+          return "device allocation: 3D work list";
+        }
     }
   }
   if (d == 2) return build_p2_level(m, level, L);

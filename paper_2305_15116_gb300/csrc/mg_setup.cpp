@@ -320,10 +320,6 @@ std::string solver_setup(Mesh& m, int max_level, int nu1, int nu2, double omega)
   const int nw = d == 2 ? NW2 : NW3;
   if (m.n_verts > 4096) return "the coarsest level has more than 4096 vertices (dense direct solve)";
   solver_free(m);
-  if (d == 3) {
-    const cudaError_t e = slab3d_prepare();  // before any captured cycle
-    if (e != cudaSuccess) return std::string("cuda: ") + cudaGetErrorString(e);
-  }
   m.solver = new Solver();
   Solver& sv = *m.solver;
   sv.max_level = max_level;

@@ -25,14 +25,14 @@ struct ModeArgs {
 // u, b and dinv of the point already in registers
 template <int MODE, class T>
 __device__ __forceinline__ T mode_out_staged(T au, T u, T b, T d, double omega) {
-  if (MODE == MODE_APPLY || MODE == MODE_PARTIAL) return au;
+  if (MODE != MODE_JACOBI && MODE != MODE_RESIDUAL) return au;
   if (MODE == MODE_RESIDUAL) return b - au;
   return u + (T)omega * d * (b - au);
 }
 
 template <int MODE, class T>
 __device__ __forceinline__ T mode_out(T au, const T* __restrict__ x, const ModeArgs& md, int64_t i) {
-  if (MODE == MODE_APPLY || MODE == MODE_PARTIAL) return au;
+  if (MODE != MODE_JACOBI && MODE != MODE_RESIDUAL) return au;
   const T bi = __ldg(static_cast<const T*>(md.b) + i);
   if (MODE == MODE_RESIDUAL) return bi - au;
   const T ui = __ldg(x + i), di = __ldg(static_cast<const T*>(md.dinv) + i);

@@ -6,7 +6,7 @@
 // The paper takes the refinement levels as the natural multigrid hierarchy
 // (Sec. 1.2) and lists smoothers among the kernels HyTeG generates (Sec. 5.1);
 // the operator apply of every smoothing step is the stencil apply of this
-// library (interior2d.cu / slab3d.cu + interface.cu).
+// library (interior2d.cu, apply3d.cu).
 //
 // Vectors are in the slot layout of their level.  Restriction works on
 // consistent fine vectors: each macro sums the fine values around each of
@@ -775,26 +775,7 @@ cudaError_t apply_g(Mesh* const* ms, int cnt, int l, int dtype, const void* cons
     if (ms[0]->dim == 2) {
       HY_TRY(launch_apply2d_batch(dt, mm.data(), lv.data(), xx.data(), yy.data(), k, s));
     } else {
-      // small vectors in one launch, the others with their interface step after it
-      for (int direct = 0; direct < 2; ++direct) {
-        std::vector<const Mesh*> md;
-        std::vector<const void*> xd;
-        std::vector<void*> yd;
-        for (int i = 0; i < k; ++i) {
-          if (int(mm[i]->levels[l].direct3) != direct) continue;
-          md.push_back(mm[i]);
-          xd.push_back(xx[i]);
-          yd.push_back(yy[i]);
-        }
-        if (md.empty()) continue;
-        const int kd = int(md.size());
-        if (direct) {
-          HY_TRY(launch_direct3d_group(dt, false, md.data(), lv.data(), xd.data(), yd.data(), kd, s));
-        } else {
-          HY_TRY(launch_slab3d_group(dt, md.data(), lv.data(), xd.data(), yd.data(), kd, s));
-          HY_TRY(launch_interface_reduce_group(dt, md.data(), lv.data(), xd.data(), yd.data(), kd, s));
-        }
-      }
+      HY_TRY(launch_apply3d_group(dt, false, mm.data(), lv.data(), xx.data(), yy.data(), k, s));
     }
   }
   return cudaSuccess;
@@ -806,8 +787,6 @@ cudaError_t accurate_g(Mesh* const* ms, int cnt, int l, const double* const* u, 
                        double* const* y, cudaStream_t s) {
   std::vector<const Mesh*> mm(ms, ms + cnt);
   std::vector<int> lv(cnt, l);
-  std::vector<const void*> uu(u, u + cnt);
-  std::vector<void*> yy(y, y + cnt);
   if (ms[0]->dim == 2) {
     Batch<PartialDiff<2>> B;
     for (int i = 0; i < cnt; ++i) {
@@ -828,7 +807,7 @@ cudaError_t accurate_g(Mesh* const* ms, int cnt, int l, const double* const* u, 
     HY_TRY(B.launch(s));
   }
   // sum the copies; Dirichlet rows: y = u
-  return launch_interface_reduce_group(3, mm.data(), lv.data(), uu.data(), yy.data(), cnt, s);
+  return launch_sum_copies(mm.data(), lv.data(), u, y, cnt, s);
 }
 
 // 2D fp32 fused sweeps (apply, interface and Jacobi update or residual in one

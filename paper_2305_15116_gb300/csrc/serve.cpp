@@ -69,18 +69,18 @@ int64_t slots_of(int dim, int level, int64_t n_cells) { return hyteg::slots_per_
 
 // Device bytes of a request: per level the solver workspace (2 inverse
 // diagonals, owner flags, 4 float64 and 4 fp32 vectors: 61 B per slot) and
-// its tables (3D: the interface slot table), plus b, u, u_lo (slot layout) and the global-order buffer on
+// its tables (3D: interface lists), plus b, u, u_lo (slot layout) and the global-order buffer on
 // the finest level, with a margin for tables and allocation rounding.
 size_t estimate_bytes(int dim, int level, int64_t n_cells, int64_t n_verts) {
   size_t b = 0;
   for (int l = 0; l <= level; ++l) {
     const int64_t S = hyteg::slots_per_macro(dim, l);
-    // 3D: + the slot and pair tables of the interface copies (about 8 B per slot)
+    // 3D: + the interface lists, weights and point tables (at most 8 B per slot)
     b += size_t(dim == 3 ? 69 : 61) * size_t(S * n_cells) + size_t(4) * size_t(S) + (size_t(64) << 10);
   }
   const int64_t ns = slots_of(dim, level, n_cells);
   b += size_t(32) * size_t(ns);
-  // 3D: scratch vectors of the slab work-split autotuner (two float64
+  // 3D: scratch vectors of the work-split autotuner (two float64
   // vectors on the levels it times, all levels together below 20 B per slot)
   if (dim == 3) b += size_t(20) * size_t(ns);
   b += size_t(8) * size_t(n_verts) * size_t(n_verts) * 2;  // dense level-0 inverse (fp64 + fp32 copy)
@@ -99,7 +99,7 @@ std::string make_key(const Req& r) {
 }
 
 // Requests solved together: at most kMaxGroup of one class.  3D levels above
-// 6 (the row kernel) have no group launch and are solved alone.
+// 6 fill the device by themselves and are solved alone.
 constexpr int kMaxGroup = 8;
 bool same_class(const Req& a, const Req& b) {
   return a.dim == b.dim && a.level == b.level && a.mode == b.mode && a.rtol == b.rtol && a.max_iter == b.max_iter;

@@ -63,7 +63,7 @@ class Mesh:
         return self
 
     def autotune_choice(self, level: int, dtype: int = F64) -> int:
-        """z-ranges per macro-tet the 3D slab autotuner picked (0: not tuned)."""
+        """What the refinement's autotuner picked: 2D rows per tile, 3D z-ranges per macro-tet (0: not tuned)."""
         v = ctypes.c_int()
         C.check(C.lib.hyteg_autotune_choice(self._h, level, dtype, ctypes.byref(v)), "hyteg_autotune_choice")
         return v.value
