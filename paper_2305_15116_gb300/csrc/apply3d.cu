@@ -258,9 +258,11 @@ cudaError_t march_attr() {
   static cudaError_t err = cudaSuccess;
   std::call_once(once, [] {
     err = cudaFuncSetAttribute(k_group<B, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::smem_bytes());
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(k_group<B, kGroupMax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)B::smem_bytes());
+    if constexpr (STRIDE <= 512) {
+      if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(k_group<B, kGroupMax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)B::smem_bytes());
+    }
   });
   return err;
 }
@@ -299,7 +301,10 @@ cudaError_t launch_march_s(const Mesh* const* ms, const int* levels, const void*
     prm.push_back(p);
     blocks.push_back(int(all));
   }
-  return launch_group<B>(prm.data(), blocks.data(), count, s, B::smem_bytes());
+  if constexpr (STRIDE <= 512) return launch_group<B>(prm.data(), blocks.data(), count, s, B::smem_bytes());
+  cudaError_t e = cudaSuccess;  // large levels fill the device each by itself
+  for (int i = 0; i < count && e == cudaSuccess; ++i) e = launch_one<B>(prm[i], blocks[i], s, B::smem_bytes());
+  return e;
 }
 
 // The slot size is a constant of the kernel: the columns of a block with their
@@ -394,6 +399,16 @@ cudaError_t launch_apply3d_group(int dtype, bool partial, const Mesh* const* ms,
   if (count <= 0) return cudaSuccess;
   return partial ? launch_dt<MODE_PARTIAL>(dtype, ms, levels, xs, ys, count, s)
                  : launch_dt<MODE_APPLY>(dtype, ms, levels, xs, ys, count, s);
+}
+
+cudaError_t launch_sweep3d_group(bool jacobi, const Mesh* const* ms, const int* levels, const void* const* u,
+                                 const void* const* b, const void* const* dinv, const double* omega,
+                                 void* const* out, int count, cudaStream_t s) {
+  if (count <= 0) return cudaSuccess;
+  std::vector<ModeArgs> md(count);
+  for (int i = 0; i < count; ++i) md[i] = ModeArgs{b[i], dinv[i], omega[i]};
+  return jacobi ? launch_t<ArF32, MODE_JACOBI>(ms, levels, u, out, md.data(), count, s)
+                : launch_t<ArF32, MODE_RESIDUAL>(ms, levels, u, out, md.data(), count, s);
 }
 
 cudaError_t launch_march3d_work(int dtype, const Mesh& m, int level, const March3Work& work, const void* x, void* y,

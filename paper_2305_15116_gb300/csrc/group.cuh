@@ -88,21 +88,25 @@ __global__ void __launch_bounds__(Body::kThreads, min_blocks<Body>::value) k_gro
   Body::run(g.p[e], (int)blockIdx.x - g.begin[e], g.begin[e + 1] - g.begin[e]);
 }
 
+// Launches Body for one mesh.
+template <class Body>
+cudaError_t launch_one(const typename Body::Prm& p, int blocks, cudaStream_t s, size_t smem = 0) {
+  if (blocks <= 0) return cudaSuccess;
+  GroupArgs<typename Body::Prm, 1> g;
+  g.p[0] = p;
+  g.begin[0] = 0;
+  g.begin[1] = blocks;
+  g.count = 1;
+  return launch_pdl(k_group<Body, 1>, dim3((unsigned)blocks), dim3(Body::kThreads), smem, s, g);
+}
+
 // Launches Body over `count` meshes, blocks[i] blocks for mesh i (meshes with
 // no blocks are skipped), in launches of at most kGroupMax meshes.
 template <class Body>
 cudaError_t launch_group(const typename Body::Prm* p, const int* blocks, int count, cudaStream_t s,
                          size_t smem = 0) {
   using Prm = typename Body::Prm;
-  if (count == 1) {
-    if (blocks[0] <= 0) return cudaSuccess;
-    GroupArgs<Prm, 1> g;
-    g.p[0] = p[0];
-    g.begin[0] = 0;
-    g.begin[1] = blocks[0];
-    g.count = 1;
-    return launch_pdl(k_group<Body, 1>, dim3((unsigned)blocks[0]), dim3(Body::kThreads), smem, s, g);
-  }
+  if (count == 1) return launch_one<Body>(p[0], blocks[0], s, smem);
   for (int i0 = 0; i0 < count;) {
     GroupArgs<Prm, kGroupMax> g;
     g.count = 0;

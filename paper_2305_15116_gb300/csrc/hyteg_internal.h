@@ -363,6 +363,10 @@ constexpr int kDirect3TableN = 128;
 // included (partial: every interface copy keeps its own macro's partial row)
 cudaError_t launch_apply3d_group(int dtype, bool partial, const Mesh* const* ms, const int* levels,
                                  const void* const* xs, void* const* ys, int count, cudaStream_t s);
+// the fp32 fused sweeps of 3D meshes (as launch_sweep2d_group)
+cudaError_t launch_sweep3d_group(bool jacobi, const Mesh* const* ms, const int* levels, const void* const* u,
+                                 const void* const* b, const void* const* dinv, const double* omega,
+                                 void* const* out, int count, cudaStream_t s);
 // the march over an explicit work list (the autotuner's candidates)
 cudaError_t launch_march3d_work(int dtype, const Mesh& m, int level, const March3Work& work, const void* x, void* y,
                                 cudaStream_t s);

@@ -810,11 +810,11 @@ cudaError_t accurate_g(Mesh* const* ms, int cnt, int l, const double* const* u, 
   return launch_sum_copies(mm.data(), lv.data(), u, y, cnt, s);
 }
 
-// 2D fp32 fused sweeps (apply, interface and Jacobi update or residual in one
+// fp32 fused sweeps (apply, interface and Jacobi update or residual in one
 // launch): out = sweep(cur) with the level's b and inverse diagonal
-cudaError_t sweep2d_g(bool jacobi, Mesh* const* ms, int cnt, int l, const float* const* cur, const float* const* b,
+cudaError_t sweep_g(bool jacobi, Mesh* const* ms, int cnt, int l, const float* const* cur, const float* const* b,
                       float* const* out, cudaStream_t s) {
-  if (cnt == 1) {
+  if (cnt == 1 && ms[0]->dim == 2) {
     const Mesh& m = *ms[0];
     return launch_sweep2d(2, jacobi, m, m.levels[l], cur[0], b[0], m.solver->lv[l].dinv32, m.solver->omega, out[0],
                           s);
@@ -828,16 +828,16 @@ cudaError_t sweep2d_g(bool jacobi, Mesh* const* ms, int cnt, int l, const float*
     dd[i] = ms[i]->solver->lv[l].dinv32;
     om[i] = ms[i]->solver->omega;
   }
-  return launch_sweep2d_group(jacobi, mm.data(), lv.data(), uu.data(), bb.data(), dd.data(), om.data(), oo.data(),
-                              cnt, s);
+  const auto launch = ms[0]->dim == 2 ? launch_sweep2d_group : launch_sweep3d_group;
+  return launch(jacobi, mm.data(), lv.data(), uu.data(), bb.data(), dd.data(), om.data(), oo.data(), cnt, s);
 }
 
-// Whether a level's sweeps are fused 2D fp32 launches (apply, interface and
+// Whether a level's sweeps are fused launches (fp32: apply, interface and
 // Jacobi update together, alternating between the level's u and y) rather
 // than an apply followed by an in-place update.
 template <class T>
-bool fused_sweeps(const Mesh& m) {
-  return sizeof(T) == 4 && m.dim == 2;
+bool fused_sweeps(const Mesh&) {
+  return sizeof(T) == 4;
 }
 
 // The vector that receives a level's first sweep from a zero guess when the
@@ -871,15 +871,15 @@ cudaError_t vcycle_g(Mesh* const* ms, int cnt, int l, const T* const* b, T* cons
     fc[i] = first_sweep_vector<T>(*ms[i], l - 1);
     if (fused && first_done) cur[i] = y[i];  // where the first sweep landed
   }
-  // 2D fp32 cycles: every sweep is one fused launch (apply, interface and
+  // fp32 cycles: every sweep is one fused launch (apply, interface and
   // Jacobi update together), alternating between u and y; the residual
-  // likewise.  Float64 cycles and 3D: apply, then update.  `cur` holds the
+  // likewise.  Float64 cycles: apply, then update.  `cur` holds the
   // smoothed iterate; it alternates between u and y and is copied back into
   // u only if the sweep count is odd.
   auto sweeps = [&](int count) -> cudaError_t {
     for (int it = 0; it < count; ++it) {
       for (int i = 0; i < cnt; ++i) alt[i] = cur[i] == u[i] ? y[i] : u[i];
-      HY_TRY(sweep2d_g(true, ms, cnt, l, reinterpret_cast<const float* const*>(cur.data()),
+      HY_TRY(sweep_g(true, ms, cnt, l, reinterpret_cast<const float* const*>(cur.data()),
                        reinterpret_cast<const float* const*>(b), reinterpret_cast<float* const*>(alt.data()), s));
       cur.swap(alt);
     }
@@ -890,7 +890,7 @@ cudaError_t vcycle_g(Mesh* const* ms, int cnt, int l, const T* const* b, T* cons
   const int pre = sv0.nu1 - (first_done ? 1 : 0);
   if (fused) {
     HY_TRY(sweeps(pre));
-    HY_TRY(sweep2d_g(false, ms, cnt, l, reinterpret_cast<const float* const*>(cur.data()),
+    HY_TRY(sweep_g(false, ms, cnt, l, reinterpret_cast<const float* const*>(cur.data()),
                      reinterpret_cast<const float* const*>(b), reinterpret_cast<float* const*>(r.data()), s));
   } else {
     for (int it = 0; it < pre; ++it) {
