@@ -13,67 +13,12 @@
 #include <type_traits>
 #include <vector>
 
+#include "direct.cuh"
 #include "march3d.cuh"
 
 namespace hyteg {
 
 namespace {
-
-// Single-point forms of the policies' pair operations, in the same order of
-// roundings, so that a point's value does not depend on the kernel that
-// computes it.
-template <class P>
-struct One;
-template <>
-struct One<ArF32> {
-  using Acc = float;
-  static __device__ __forceinline__ void first(Acc& a, const float& w, float v) { a = __fmul_rn(w, v); }
-  static __device__ __forceinline__ void sym(Acc& a, const float& w, float u, float v) {
-    a = __fmaf_rn(w, __fadd_rn(u, v), a);
-  }
-  static __device__ __forceinline__ float finish(Acc a) { return a; }
-  static __device__ __forceinline__ bool bad(Acc) { return false; }
-};
-template <>
-struct One<ArF64Native> {
-  using Acc = double;
-  static __device__ __forceinline__ void first(Acc& a, const double& w, double v) { a = __dmul_rn(w, v); }
-  static __device__ __forceinline__ void sym(Acc& a, const double& w, double u, double v) {
-    a = __fma_rn(w, __dadd_rn(u, v), a);
-  }
-  static __device__ __forceinline__ double finish(Acc a) { return a; }
-  static __device__ __forceinline__ bool bad(Acc) { return false; }
-};
-template <>
-struct One<ArF64FF> {
-  struct Acc {
-    float s, e;
-  };
-  static __device__ __forceinline__ void first(Acc& a, const ArF64FF::W& w, FF v) {
-    const float pm = __fmul_rn(-w.h1, v.h);
-    a.s = __fsub_rn(0.0f, pm);
-    float e = __fmaf_rn(w.h1, v.h, pm);
-    e = __fmaf_rn(w.h1, v.l, e);
-    a.e = __fmaf_rn(w.l1, v.h, e);
-  }
-  static __device__ __forceinline__ void sym(Acc& a, const ArF64FF::W& w, FF u, FF v) {
-    const float sh = __fadd_rn(u.h, v.h);
-    const float bb = __fsub_rn(sh, u.h);
-    const float er = __fadd_rn(__fsub_rn(u.h, __fsub_rn(sh, bb)), __fsub_rn(v.h, bb));
-    const float sl = __fadd_rn(__fadd_rn(u.l, v.l), er);
-    float e = __fmaf_rn(w.h1, sl, a.e);
-    const float pm = __fmul_rn(-w.h1, sh);
-    e = __fmaf_rn(w.l1, sh, e);
-    const float sn = __fsub_rn(a.s, pm);
-    const float nbp = __fsub_rn(a.s, sn);
-    const float t2 = __fsub_rn(a.s, __fadd_rn(sn, nbp));
-    a.s = sn;
-    e = __fadd_rn(e, __fmaf_rn(w.h1, sh, nbp));
-    a.e = __fadd_rn(e, t2);
-  }
-  static __device__ __forceinline__ double finish(const Acc& a) { return ff_join(a.s, a.e); }
-  static __device__ __forceinline__ bool bad(const Acc& a) { return a.s != a.s; }
-};
 
 template <class P, int MODE>
 struct Direct3 {
@@ -104,42 +49,16 @@ struct Direct3 {
     if (t >= p.n_pts) return;
     const int2 e = p.pts[t];
     const int64_t wb = (int64_t)m * (NCLS3 * NW3);
-    const typename P::W w0 = P::weight(p.st, wb), w1 = P::weight(p.st, wb + 1), w3 = P::weight(p.st, wb + 3),
-                        w5 = P::weight(p.st, wb + 5), w7 = P::weight(p.st, wb + 7), w8 = P::weight(p.st, wb + 8),
-                        w9 = P::weight(p.st, wb + 9), w10 = P::weight(p.st, wb + 10);
+    InnerW<3, P> W;
+    W.load(p.st, wb);
     const Off15 o(e.y >> 16, e.y & 0xFFFF);
     const int64_t i = (int64_t)m * p.S + e.x;
-    const T* __restrict__ xp = p.x + i;
     pdl_wait();
-    T v[NW3];
-#pragma unroll
-    for (int k = 0; k < NW3; ++k) v[k] = __ldg(xp + o[k]);
-    T bi = T(0), di = T(0);
-    if (MODE == MODE_JACOBI || MODE == MODE_RESIDUAL) bi = __ldg(static_cast<const T*>(p.md.b) + i);
+    T bi = T(0), di = T(0), uc;
+    if (MODE == MODE_JACOBI || MODE == MODE_RESIDUAL) bi = ld<false>(static_cast<const T*>(p.md.b) + i);
     if (MODE == MODE_JACOBI) di = __ldg(static_cast<const T*>(p.md.dinv) + i);
-    using O = One<P>;
-    typename O::Acc a;
-    O::first(a, w0, P::conv(v[0]));
-    O::sym(a, w1, P::conv(v[1]), P::conv(v[2]));
-    O::sym(a, w3, P::conv(v[3]), P::conv(v[4]));
-    O::sym(a, w5, P::conv(v[5]), P::conv(v[6]));
-    O::sym(a, w7, P::conv(v[7]), P::conv(v[11]));
-    O::sym(a, w8, P::conv(v[8]), P::conv(v[12]));
-    O::sym(a, w9, P::conv(v[9]), P::conv(v[13]));
-    O::sym(a, w10, P::conv(v[10]), P::conv(v[14]));
-    T r = O::finish(a);
-    if constexpr (P::kPoison) {  // an input outside the float-float range: native fp64 row
-      if (O::bad(a)) {
-        const double* __restrict__ wd = p.st.d + wb;
-        r = 0.0;
-#pragma unroll
-        for (int k = 0; k < NW3; ++k) {
-          const double wk = __ldg(wd + k);
-          if (wk != 0.0) r = __fma_rn(wk, v[k], r);
-        }
-      }
-    }
-    p.y[i] = mode_out_staged<MODE, T>(r, v[0], bi, di, p.md.omega);
+    const T r = inner_row<3, P, false>(p.x + i, o, W, p.st, wb, uc);
+    p.y[i] = mode_out_staged<MODE, T>(r, uc, bi, di, p.md.omega);
   }
 };
 
@@ -157,12 +76,12 @@ const float* face_table<float>(const LevelDev& L) {
 template <class T>
 Iface3<T> iface_of(const Mesh& m, const LevelDev& L) {
   Iface3<T> f;
-  f.items = L.if3;
-  f.n_items = L.n_if3_ev;
+  f.items = L.ifi;
+  f.n_items = L.n_ifi_ev;
   f.per_face = std::max(1, (L.n_face_pts + 31) / 32);
   f.n_pts = L.n_face_pts;
   f.n_faces = L.n_face3;
-  f.n_units = L.n_if3_ev + f.per_face * L.n_face3;
+  f.n_units = L.n_ifi_ev + f.per_face * L.n_face3;
   f.faces = L.face3;
   f.ab = L.face_ab;
   f.incs = m.d_incs;
@@ -376,7 +295,7 @@ struct Sum3 {
   struct Prm {
     const T* x;
     T* y;
-    const If3Item* items;
+    const IfItem* items;
     int n_items;
     const Inc* incs;
     int n;
@@ -385,10 +304,13 @@ struct Sum3 {
   static __device__ __forceinline__ void run(const Prm& p, int block, int) {
     const int item = (kThreads / 32) * block + (int)(threadIdx.x >> 5);
     if (item >= p.n_items) return;
-    const If3Item it = p.items[item];
+    const IfItem it = p.items[item];
     pdl_wait();
-    iface3d_item<MODE_SUM, false, T>(p.x, p.y, it.work, (int)(threadIdx.x & 31), it.prim, p.incs, p.n, p.S, StencilPtr{},
-                                     ModeArgs{});
+    run_item<3, false, T>(
+        it.work, (int)(threadIdx.x & 31), it.prim, p.incs, p.n, p.S,
+        [&](int cell, const Pt<3>& q) { return p.y[(int64_t)cell * p.S + q.slot]; },
+        [&](int64_t s) { return ld<false>(p.x + s); }, [&](T a, int64_t) { return a; },
+        [&](int64_t s, T v) { p.y[s] = v; });
   }
 };
 
@@ -429,8 +351,8 @@ cudaError_t launch_sum_copies3d(const Mesh* const* ms, const int* levels, const 
   std::vector<int> blocks;
   for (int i = 0; i < count; ++i) {
     const LevelDev& L = ms[i]->levels[levels[i]];
-    prm.push_back({xs[i], ys[i], L.if3, L.n_if3, ms[i]->d_incs, L.n, L.slots_per_macro});
-    blocks.push_back((L.n_if3 + B::kThreads / 32 - 1) / (B::kThreads / 32));
+    prm.push_back({xs[i], ys[i], L.ifi, L.n_ifi, ms[i]->d_incs, L.n, L.slots_per_macro});
+    blocks.push_back((L.n_ifi + B::kThreads / 32 - 1) / (B::kThreads / 32));
   }
   return launch_group<B>(prm.data(), blocks.data(), count, s);
 }

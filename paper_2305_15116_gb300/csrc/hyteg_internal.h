@@ -35,9 +35,9 @@ struct Prim {
   int inc_count;   // number of incident cells (ascending cell id)
 };
 
-// Item of the 3D interface work list: (-, first point, points, lanes per
-// point) of one primitive.
-struct If3Item {
+// Interface work item: (-, first point, points, lanes per point) of one
+// primitive.
+struct IfItem {
   int4 work;
   Prim prim;
 };
@@ -84,12 +84,10 @@ struct LevelDev {
   // interface work list: int4 (prim, b, a0, a1)
   int4* items = nullptr;
   int n_items = 0;
-  // 3D: interface work list of the one-launch apply, int4 (prim, first
-  // point, points, lanes per point)
-  // first the edges and vertices (n_if3_ev items), then the faces, which the
-  // apply takes from face3 instead
-  If3Item* if3 = nullptr;
-  int n_if3 = 0, n_if3_ev = 0;
+  // interface work items (lattice.cuh): first the vertices and edges (n_ifi_ev
+  // items), then in 3D the faces, which the apply takes from face3 instead
+  IfItem* ifi = nullptr;
+  int n_ifi = 0, n_ifi_ev = 0;
   Face3Rec* face3 = nullptr;
   int n_face3 = 0, n_face_pts = 0;
   unsigned* face_ab = nullptr;  // interior points of a face, a | b << 16

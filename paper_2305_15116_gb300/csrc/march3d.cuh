@@ -416,8 +416,8 @@ struct March3 {
       }
       if constexpr (kSweep) {
         if (s >= zlo && s <= zhi) {
-          ba = __ldg(bpa);
-          bb = __ldg(bpb);
+          ba = ld<false>(bpa);
+          bb = ld<false>(bpb);
         }
         bpa += c_now - (n + 1 - s);
         bpb += c_now - (n + 1 - s);

@@ -327,7 +327,7 @@ void free_level(const Mesh& m, LevelDev& L) {
   dev_free(m, L.items);
   for (int t = 0; t < 4; ++t) dev_free(m, L.march[t].work);
   dev_free(m, L.pts3);
-  dev_free(m, L.if3);
+  dev_free(m, L.ifi);
   dev_free(m, L.face3);
   dev_free(m, L.face_ab);
   dev_free(m, L.wf64);
@@ -528,22 +528,24 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
   if (!(err = upload(m, &L.tiles, tiles)).empty()) return err;
   if (!(err = upload(m, &L.tiles32, tiles32)).empty()) return err;
   if (!(err = upload(m, &L.items, items)).empty()) return err;
-  if (d == 3) {
-    // interface work list of the 3D apply (iface3d.cuh): (prim, first point,
-    // points, lanes per point), one warp per item
-    std::vector<If3Item> if3;
-    for (size_t p = 0; p < m.prims.size(); ++p) {
-      const Prim& pr = m.prims[p];
+  {
+    // interface work items (lattice.cuh): (-, first point, points, lanes per
+    // point), one warp per item; vertices, edges, then (3D) faces
+    std::vector<IfItem> ifi;
+    for (const Prim& pr : m.prims) {
       const int64_t np = pr.type == 0 ? 1 : pr.type == 1 ? n - 1 : int64_t(n - 1) * (n - 2) / 2;
       int lanes = 1;
       if (pr.inc_count > 2 && pr.inc_count <= 32 && !pr.boundary)
         while (lanes < pr.inc_count) lanes *= 2;
       const int per = 32 / lanes;
       for (int64_t t = 0; t < np; t += per)
-        if3.push_back({make_int4(int(p), int(t), int(std::min<int64_t>(per, np - t)), lanes), pr});
+        ifi.push_back({make_int4(0, int(t), int(std::min<int64_t>(per, np - t)), lanes), pr});
     }
-    L.n_if3 = int(if3.size());
-    L.n_if3_ev = int(std::count_if(if3.begin(), if3.end(), [](const If3Item& i) { return i.prim.type < 2; }));
+    L.n_ifi = int(ifi.size());
+    L.n_ifi_ev = int(std::count_if(ifi.begin(), ifi.end(), [](const IfItem& i) { return i.prim.type < 2; }));
+    if (!(err = upload(m, &L.ifi, ifi)).empty()) return err;
+  }
+  if (d == 3) {
     std::vector<unsigned> ab;
     for (int b = 1; b <= n - 2; ++b)
       for (int a = 1; a <= n - 1 - b; ++a) ab.push_back(unsigned(a) | unsigned(b) << 16);
@@ -576,7 +578,6 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     L.n_face_pts = int(ab.size());
     if (!(err = upload(m, &L.face3, faces)).empty()) return err;
     if (!(err = upload(m, &L.face_ab, ab)).empty()) return err;
-    if (!(err = upload(m, &L.if3, if3)).empty()) return err;
     // the face without corner f is x+y+z = n (f = 0) or x, y, z = 0
     std::vector<double> wf(size_t(m.n_cells) * 4 * 12, 0.0);
     for (int64_t c = 0; c < m.n_cells; ++c)

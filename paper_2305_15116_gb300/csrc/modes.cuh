@@ -22,21 +22,42 @@ struct ModeArgs {
 };
 
 #ifdef __CUDACC__
+// A load of a vector's value: a plain one, or (CG) from L2, where values
+// written by other blocks of the same launch are seen after a barrier between
+// them.  Not the read-only path: a kernel may start before the one that writes
+// the vector has finished (group.cuh), and the code generator may move a
+// read-only load, which it takes for invariant, above the wait.
+template <bool CG, class T>
+__device__ __forceinline__ T ld(const T* p) {
+  if constexpr (CG)
+    return __ldcg(p);
+  else
+    return *p;
+}
+
+__device__ __forceinline__ float jacobi_out(float au, float u, float b, float d, float omega) {
+  return __fmaf_rn(__fmul_rn(omega, d), __fsub_rn(b, au), u);
+}
+__device__ __forceinline__ double jacobi_out(double au, double u, double b, double d, double omega) {
+  return __fma_rn(__dmul_rn(omega, d), __dsub_rn(b, au), u);
+}
 // u, b and dinv of the point already in registers
 template <int MODE, class T>
 __device__ __forceinline__ T mode_out_staged(T au, T u, T b, T d, double omega) {
   if (MODE != MODE_JACOBI && MODE != MODE_RESIDUAL) return au;
   if (MODE == MODE_RESIDUAL) return b - au;
-  return u + (T)omega * d * (b - au);
+  return jacobi_out(au, u, b, d, (T)omega);
 }
 
-template <int MODE, class T>
-__device__ __forceinline__ T mode_out(T au, const T* __restrict__ x, const ModeArgs& md, int64_t i) {
+// CG: loads from L2 (vectors written earlier in the same launch)
+template <int MODE, bool CG, class T>
+__device__ __forceinline__ T mode_out(T au, const T* x, const ModeArgs& md, int64_t i) {
   if (MODE != MODE_JACOBI && MODE != MODE_RESIDUAL) return au;
-  const T bi = __ldg(static_cast<const T*>(md.b) + i);
+  const T* const bp = static_cast<const T*>(md.b) + i;
+  const T bi = ld<CG>(bp);
   if (MODE == MODE_RESIDUAL) return bi - au;
-  const T ui = __ldg(x + i), di = __ldg(static_cast<const T*>(md.dinv) + i);
-  return ui + (T)md.omega * di * (bi - au);
+  const T ui = ld<CG>(x + i), di = __ldg(static_cast<const T*>(md.dinv) + i);
+  return jacobi_out(au, ui, bi, di, (T)md.omega);
 }
 #endif
 

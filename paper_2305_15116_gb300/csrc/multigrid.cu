@@ -18,9 +18,7 @@
 #include <cmath>
 #include <vector>
 
-#include "arith.cuh"
-#include "group.cuh"
-#include "hyteg_internal.h"
+#include "transfer.cuh"
 
 namespace hyteg {
 
@@ -68,10 +66,6 @@ __constant__ int c_off2[NW2][2] = {{0, -1}, {1, -1}, {-1, 0}, {0, 0}, {1, 0}, {-
 __constant__ int c_off3[NW3][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0},
                                    {1, -1, 0}, {-1, 1, 0}, {0, 0, 1},  {-1, 0, 1}, {0, -1, 1},
                                    {1, -1, 1}, {0, 0, -1}, {1, 0, -1}, {0, 1, -1}, {-1, 1, -1}};
-
-// micro-edge directions of the refinement (2D triangles, 3D Kuhn tets)
-__constant__ int c_dir2[3][2] = {{1, 0}, {0, 1}, {1, -1}};
-__constant__ int c_dir3[7][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {1, -1, 0}, {1, 0, -1}, {0, 1, -1}, {1, -1, 1}};
 
 // ---- kernel bodies ----------------------------------------------------------------
 // Every kernel the solve loop and the V-cycle launch is a body run by
@@ -240,40 +234,6 @@ struct PartialDiff {
 
 // ---- transfers --------------------------------------------------------------
 
-// One macro's partial of (P^T r) at its coarse point q: the fine value at the
-// coincident point plus half the values at the midpoints of the coarse
-// micro-edges around it (6 in 2D, 14 in 3D), each divided by the number of
-// macros holding a copy of it (a per-macro table by boundary class).
-template <class T, int DIM>
-__device__ __forceinline__ T restrict_partial(const T* __restrict__ rf, const T* __restrict__ multinv, int64_t cell,
-                                              const int q[3], int nc, int64_t Sf) {
-  constexpr int NCLS = DIM == 2 ? NCLS2 : NCLS3;
-  constexpr int ND = DIM == 2 ? 3 : 7;
-  const int nf = 2 * nc;
-  const int f[3] = {2 * q[0], 2 * q[1], 2 * q[2]};
-  const T* __restrict__ r = rf + cell * Sf;
-  const T* __restrict__ mi = multinv + cell * NCLS;
-  T acc = r[slotq<DIM>(nf, f)] * mi[pclass<DIM>(nf, f)];
-#pragma unroll
-  for (int k = 0; k < ND; ++k) {
-#pragma unroll
-    for (int sgn = -1; sgn <= 1; sgn += 2) {
-      int j[3];
-      if (DIM == 2) {
-        j[0] = f[0] + sgn * c_dir2[k][0];
-        j[1] = f[1] + sgn * c_dir2[k][1];
-        j[2] = 0;
-      } else {
-        j[0] = f[0] + sgn * c_dir3[k][0];
-        j[1] = f[1] + sgn * c_dir3[k][1];
-        j[2] = f[2] + sgn * c_dir3[k][2];
-      }
-      if (inside<DIM>(nf, j)) acc += T(0.5) * r[slotq<DIM>(nf, j)] * mi[pclass<DIM>(nf, j)];
-    }
-  }
-  return acc;
-}
-
 // b_c = P^T r_f in one launch: blocks [0, n_if_blocks) take the coarse
 // interface items (each point sums the partials of its copies in ascending
 // macro order and writes every copy; Dirichlet points get 0), the others the
@@ -291,8 +251,8 @@ struct Restrict {
     T omega;
     const unsigned* lpts_c;
     const T* multinv;
-    const int4* items;
-    const Prim* prims;
+    const IfItem* items;
+    int n_items;
     const Inc* incs;
     int nc;
     int64_t Sc, Sf, total;
@@ -300,84 +260,37 @@ struct Restrict {
   };
   static __device__ __forceinline__ void run(const Prm& p, int block, int nb) {
     const int nc = p.nc;
+    auto row = [&](int64_t cell, const Pt<DIM>& q) {
+      return restrict_row<DIM, false>(p.rf + cell * p.Sf, p.multinv + cell * Lat<DIM>::NCLS, q, 2 * nc);
+    };
+    auto put = [&](int64_t s, T v) {
+      p.bc[s] = v;
+      if (p.uc) p.uc[s] = i3_mul(i3_mul(p.omega, __ldg(p.dinv + s)), v);
+    };
     if (block < p.n_if_blocks) {
-      const int4 it = p.items[block];
-      const Prim pr = p.prims[it.x];
+      const int k = block * (kThreads / 32) + (int)(threadIdx.x >> 5);
+      if (k >= p.n_items) return;
+      const IfItem it = p.items[k];
       pdl_wait();
-      if (pr.type == 0 && !pr.boundary && pr.inc_count <= 32) {
-        // a coarse vertex inside the domain: lane i of the first warp takes
-        // copy i, and every lane adds the partials in ascending copy order
-        // (the order of the loop below) through shuffles
-        if (threadIdx.x >= 32) return;
-        const int lane = threadIdx.x;
-        const bool mine = lane < pr.inc_count;
-        int64_t sl = 0;
-        T part = T(0);
-        if (mine) {
-          const Inc inc = p.incs[pr.inc_begin + lane];
-          int q[3] = {0, 0, 0};
-          if (inc.corner[0] >= 1) q[inc.corner[0] - 1] += nc;
-          sl = (int64_t)inc.cell * p.Sc + slotq<DIM>(nc, q);
-          part = restrict_partial<T, DIM>(p.rf, p.multinv, inc.cell, q, nc, p.Sf);
-        }
-        T acc = T(0);
-        for (int i = 0; i < pr.inc_count; ++i) acc += __shfl_sync(0xFFFFFFFFu, part, i);
-        if (mine) {
-          p.bc[sl] = acc;
-          if (p.uc) p.uc[sl] = p.omega * p.dinv[sl] * acc;
-        }
-        return;
-      }
-      const int a = it.z + threadIdx.x;
-      if (a >= it.w) return;
-      const int b = it.y;
-      int wv[3] = {0, 0, 0};
-      if (pr.type == 0) {
-        wv[0] = nc;
-      } else if (pr.type == 1) {
-        wv[0] = nc - a;
-        wv[1] = a;
-      } else {
-        wv[0] = nc - a - b;
-        wv[1] = a;
-        wv[2] = b;
-      }
-      auto local = [&](const Inc& inc, int q[3]) {
-        q[0] = q[1] = q[2] = 0;
-        for (int j = 0; j <= pr.type; ++j)
-          if (inc.corner[j] >= 1) q[inc.corner[j] - 1] += wv[j];
-      };
-      T acc = T(0);
-      if (!pr.boundary) {
-        for (int i = 0; i < pr.inc_count; ++i) {
-          const Inc inc = p.incs[pr.inc_begin + i];
-          int q[3];
-          local(inc, q);
-          acc += restrict_partial<T, DIM>(p.rf, p.multinv, inc.cell, q, nc, p.Sf);
-        }
-      }
-      for (int i = 0; i < pr.inc_count; ++i) {
-        const Inc inc = p.incs[pr.inc_begin + i];
-        int q[3];
-        local(inc, q);
-        const int64_t sl = (int64_t)inc.cell * p.Sc + slotq<DIM>(nc, q);
-        p.bc[sl] = acc;
-        if (p.uc) p.uc[sl] = p.omega * p.dinv[sl] * acc;
-      }
+      run_item<DIM, false, T>(
+          it.work, (int)(threadIdx.x & 31), it.prim, p.incs, nc, p.Sc, row, [](int64_t) { return T(0); },
+          [](T a, int64_t) { return a; }, put);
       return;
     }
-    pdl_wait();
     const SlotDiv divSc(p.Sc, p.total);
-    const int64_t stride = (int64_t)(nb - p.n_if_blocks) * 128;
-    for (int64_t i = (int64_t)(block - p.n_if_blocks) * 128 + threadIdx.x; i < p.total; i += stride) {
+    const int64_t stride = (int64_t)(nb - p.n_if_blocks) * kThreads;
+    bool waited = false;
+    for (int64_t i = (int64_t)(block - p.n_if_blocks) * kThreads + threadIdx.x; i < p.total; i += stride) {
       const int64_t cell = divSc(i);
-      int q[3];
-      unpack<DIM>(p.lpts_c[i - cell * p.Sc], q);
-      if (pclass<DIM>(nc, q) != 0) continue;  // macro-boundary point: an interface item's
-      const T acc = restrict_partial<T, DIM>(p.rf, p.multinv, cell, q, nc, p.Sf);
-      p.bc[i] = acc;
-      if (p.uc) p.uc[i] = p.omega * p.dinv[i] * acc;
+      Pt<DIM> q;
+      unpack<DIM>(p.lpts_c[i - cell * p.Sc], q.q);
+      if (pclass<DIM>(nc, q.q) != 0) continue;  // macro-boundary point: an interface item's
+      q.set(nc);
+      if (!waited) pdl_wait();
+      waited = true;
+      put(i, row(cell, q));
     }
+    if (!waited) pdl_wait();
   }
 };
 
@@ -468,32 +381,14 @@ struct Prolong {
       const int64_t cell = divSf(i);
       int q[3];
       unpack<DIM>(p.lpts_f[i - cell * p.Sf], q);
-      const T* __restrict__ e = p.ec + cell * p.Sc;
-      const int px = q[0] & 1, py = q[1] & 1, pz = q[2] & 1;
-      T v;
-      if (!(px | py | pz)) {
-        const int c[3] = {q[0] >> 1, q[1] >> 1, q[2] >> 1};
-        v = e[slotq<DIM>(nc, c)];
-      } else {
-        int d[3] = {px, py, pz};
-        if (DIM == 2) {
-          if (px && py) d[1] = -1;  // the diagonal (1,-1)
-        } else {
-          if (px && py && !pz) d[1] = -1;        // (1,-1,0)
-          else if (px && pz && !py) d[2] = -1;   // (1,0,-1)
-          else if (py && pz && !px) d[2] = -1;   // (0,1,-1)
-          else if (px && py && pz) d[1] = -1;    // (1,-1,1)
-        }
-        const int c1[3] = {(q[0] - d[0]) >> 1, (q[1] - d[1]) >> 1, (q[2] - d[2]) >> 1};
-        const int c2[3] = {(q[0] + d[0]) >> 1, (q[1] + d[1]) >> 1, (q[2] + d[2]) >> 1};
-        v = T(0.5) * (e[slotq<DIM>(nc, c1)] + e[slotq<DIM>(nc, c2)]);
-      }
+      const T v = prolong_value<DIM, false>(p.ec + cell * p.Sc, q, nc);
       p.uf[i] = p.uf[i] + v;
     }
   }
 };
 
-// Level 0: e = A0^{-1} r on the coarse vertices, written to every copy.
+// Level 0: e = A0^{-1} r on the coarse vertices, written to every copy.  Every
+// block stages the right-hand side (a gather) before it sums over the vertices.
 template <class T>
 struct Coarse {
   static constexpr int kThreads = THREADS;
@@ -505,11 +400,23 @@ struct Coarse {
     int64_t nslots;
   };
   static __device__ __forceinline__ void run(const Prm& p, int block, int nb) {
-    GRID_STRIDE(s, p.nslots) {
-      const T* __restrict__ row = p.a0inv + (int64_t)p.v_of_slot[s] * p.V;
+    __shared__ T sh[THREADS];
+    for (int64_t s0 = (int64_t)block * THREADS; s0 < p.nslots; s0 += (int64_t)nb * THREADS) {
+      const int64_t s = s0 + threadIdx.x;
+      const bool live = s < p.nslots;
+      const T* __restrict__ row = p.a0inv + (int64_t)(live ? p.v_of_slot[s] : 0) * p.V;
       T acc = T(0);
-      for (int j = 0; j < p.V; ++j) acc += row[j] * p.r[p.slot_of_v[j]];
-      p.e[s] = acc;
+      for (int j0 = 0; j0 < p.V; j0 += THREADS) {
+        const int cnt = min(THREADS, p.V - j0);
+        __syncthreads();
+        if ((int)threadIdx.x < cnt) sh[threadIdx.x] = p.r[p.slot_of_v[j0 + threadIdx.x]];
+        __syncthreads();
+        if (live) {
+#pragma unroll 8
+          for (int j = 0; j < cnt; ++j) acc = i3_fma(__ldg(row + j0 + j), sh[j], acc);
+        }
+      }
+      if (live) p.e[s] = acc;
     }
   }
 };
@@ -662,9 +569,10 @@ cudaError_t restrict_d(Mesh* const* ms, int cnt, int lf, const T* const* rf, T* 
     const MgLevel& gc = sv.lv[lf - 1];
     const int64_t want = (total + 127) / 128;
     const int int_blocks = int(want < 152 * 32 ? (want > 0 ? want : 1) : 152 * 32);
+    const int if_blocks = (Lc.n_ifi + 3) / 4;  // a warp per item
     B.add({rf[i], bc[i], uc ? uc[i] : nullptr, Vecs<T>::dinv(gc), T(sv.omega), gc.lpts, Vecs<T>::multinv(gc),
-           Lc.items, m.d_prims, m.d_incs, Lc.n, Lc.slots_per_macro, Lf.slots_per_macro, total, Lc.n_items},
-          Lc.n_items + int_blocks);
+           Lc.ifi, Lc.n_ifi, m.d_incs, Lc.n, Lc.slots_per_macro, Lf.slots_per_macro, total, if_blocks},
+          if_blocks + int_blocks);
   }
   return B.launch(s);
 }
