@@ -173,11 +173,24 @@ struct MgLevel {
   float *u32 = nullptr, *b32 = nullptr, *y32 = nullptr, *r32 = nullptr;
 };
 
+// A level as the coarse-cycle kernel sees it (coarse.cu).
+struct CoarseLev {
+  float *u, *b, *y, *r;
+  const float *dinv, *multinv, *st;
+  const unsigned* lpts;
+  const IfItem* ifi;
+  int n_ifi, n_inner, n, S;
+};
+
 struct Solver {
   int max_level = -1;
   int nu1 = 3, nu2 = 3;
   double omega = 2.0 / 3.0;
   std::vector<MgLevel> lv;
+  // device copy of the levels for the coarse-cycle kernel, and the finest level
+  // whose cycles it takes (-1: none)
+  CoarseLev* coarse = nullptr;
+  int coarse_top = -1;
   int nv0 = 0;                   // coarse (level 0) vertices
   double* a0inv64 = nullptr;     // [nv0 * nv0] inverse of the level-0 operator
   float* a0inv32 = nullptr;
@@ -322,6 +335,15 @@ void compute_lumped_mass(const Mesh& m, int level, double* mass);
 void compute_dirichlet_mask(const Mesh& m, int level, unsigned char* mask);
 std::string solver_setup(Mesh& m, int max_level, int nu1, int nu2, double omega);
 void solver_free(Mesh& m);
+// The fp32 V-cycle from level l down to level 0 and back for every member in
+// one launch, l <= Solver::coarse_top (coarse.cu); vectors as vcycle_g.
+cudaError_t launch_coarse_cycle(Mesh* const* ms, int cnt, int l, const float* const* b, float* const* u,
+                                bool first_done, cudaStream_t s);
+void coarse_cycle_prepare();  // before any stream capture
+// 2D levels of at most so many slots (one V-cycle on 32 macro-triangles at level
+// 10: 781 us without, 757, 734 and 723 us with a limit of 4000, 16000 and 32000
+// slots; with 1024 threads per block 64000 was 10 % slower than 32000)
+constexpr int64_t kCoarseMaxSlots = 32768;
 // inverse diagonals (fp64, fp32) and owner flags of one level, on the device
 cudaError_t mg_diag_setup(const Mesh& m, int level, MgLevel& g, cudaStream_t s);
 cudaError_t mg_restrict(const Mesh& m, int fine_level, int dtype, const void* rf, void* bc, cudaStream_t s);

@@ -310,6 +310,7 @@ void solver_free(Mesh& m) {
   dev_free(m, sv.v_of_slot0);
   dev_free(m, sv.slot_of_v0);
   dev_free(m, sv.red);
+  dev_free(m, sv.coarse);
   delete m.solver;
   m.solver = nullptr;
 }
@@ -472,6 +473,21 @@ std::string solver_setup(Mesh& m, int max_level, int nu1, int nu2, double omega)
   if (!(err = upload_vec(m, &sv.v_of_slot0, v_of_slot)).empty()) return err;
   if (!(err = upload_vec(m, &sv.slot_of_v0, slot_of_v)).empty()) return err;
   if (!(err = alloc_vec(m, &sv.red, size_t(1024 + 8))).empty()) return err;
+  // the levels of the coarse-cycle kernel
+  std::vector<CoarseLev> cl;
+  for (int l = 0; d == 2 && l <= max_level; ++l) {
+    const LevelDev& L = m.levels[l];
+    if (L.slots_per_macro * m.n_cells > kCoarseMaxSlots) break;
+    const MgLevel& g = sv.lv[l];
+    const int n = L.n;
+    cl.push_back({g.u32, g.b32, g.y32, g.r32, g.dinv32, g.multinv32, L.st32, g.lpts, L.ifi, L.n_ifi,
+                  n > 2 ? (n - 1) * (n - 2) / 2 : 0, n, int(L.slots_per_macro)});
+    sv.coarse_top = l;
+  }
+  if (!cl.empty()) {
+    if (!(err = upload_vec(m, &sv.coarse, cl)).empty()) return err;
+    coarse_cycle_prepare();
+  }
   const cudaError_t e = dev_sync(m);
   if (e != cudaSuccess) return std::string("cuda: set-up: ") + cudaGetErrorString(e);
   return "";

@@ -765,6 +765,11 @@ T* first_sweep_vector(Mesh& m, int l) {
 template <class T>
 cudaError_t vcycle_g(Mesh* const* ms, int cnt, int l, const T* const* b, T* const* u, cudaStream_t s,
                      bool first_done) {
+  if constexpr (sizeof(T) == 4) {  // the coarse levels in one launch
+    bool all = true;
+    for (int i = 0; i < cnt; ++i) all = all && l <= ms[i]->solver->coarse_top;
+    if (all) return launch_coarse_cycle(ms, cnt, l, b, u, first_done, s);
+  }
   if (l == 0) return coarse_g<T>(ms, cnt, u, b, s);
   const Solver& sv0 = *ms[0]->solver;
   const bool fused = fused_sweeps<T>(*ms[0]);
