@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import ctypes
+from array import array
 
 import numpy as np
 
@@ -15,10 +16,32 @@ def version() -> str:
     return C.lib.hyteg_version().decode()
 
 
+_torch = None  # set on first use: the package imports without loading torch
+_current_stream = None
+
+
+def _load_torch():
+    """torch, with the call that gives the current stream's raw handle: torch's
+    own binding where it has it (about 0.2 us), else through a Stream object
+    (about 2 us, a quarter of a small apply)."""
+    global _torch, _current_stream
+    if _torch is None:
+        import torch
+        try:
+            raw, dev = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+            _current_stream = lambda: raw(dev())
+        except AttributeError:
+            _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+        _torch = torch
+    return _torch
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _torch is None:
+            _load_torch()
+        _torch.cuda.init()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -45,6 +68,7 @@ class Mesh:
                 "hyteg_mesh_create")
         self._h = h
         self.max_level = -1
+        self._n_slots = {}  # level -> slots (they follow from the cells and the level alone)
 
     def close(self) -> None:
         if getattr(self, "_h", None):
@@ -74,6 +98,12 @@ class Mesh:
         C.check(C.lib.hyteg_num_slots(self._h, level, ctypes.byref(ns), ctypes.byref(ng)), "hyteg_num_slots")
         return ns.value, ng.value
 
+    def _slots(self, level: int) -> int:
+        n = self._n_slots.get(level)
+        if n is None:
+            n = self._n_slots[level] = self.num_slots(level)[0]
+        return n
+
     def dof_map(self, level: int) -> np.ndarray:
         """Global vertex id of every slot (int64 [n_slots])."""
         ns, _ = self.num_slots(level)
@@ -83,12 +113,13 @@ class Mesh:
 
     @staticmethod
     def _dtype_code(t, ieee: bool) -> int:
-        import torch
-        if t.dtype == torch.float32:
+        torch = _torch or _load_torch()
+        dt = t.dtype
+        if dt is torch.float32:
             return F32
-        if t.dtype == torch.float64:
+        if dt is torch.float64:
             return F64_IEEE if ieee else F64
-        raise TypeError(f"unsupported dtype {t.dtype}")
+        raise TypeError(f"unsupported dtype {dt}")
 
     def apply(self, level: int, x, y, ieee: bool = False, stream=None):
         """y = A x for device tensors x, y (float64 or float32) in slot layout.
@@ -98,13 +129,13 @@ class Mesh:
             raise ValueError("x and y must be CUDA tensors; use apply_host for host buffers")
         if x.dtype != y.dtype or not x.is_contiguous() or not y.is_contiguous():
             raise ValueError("x and y must be contiguous and of the same dtype")
-        ns, _ = self.num_slots(level)
+        ns = self._slots(level)
         if x.numel() != ns or y.numel() != ns:
             raise ValueError(f"x and y must have {ns} elements")
         code = self._dtype_code(x, ieee)
-        C.check(C.lib.hyteg_apply(self._h, level, code, ctypes.c_void_p(x.data_ptr()),
-                                  ctypes.c_void_p(y.data_ptr()), ctypes.c_void_p(_stream_ptr(stream))),
-                "hyteg_apply")
+        r = C.lib.hyteg_apply(self._h, level, code, x.data_ptr(), y.data_ptr(), _stream_ptr(stream))
+        if r:
+            C.check(r, "hyteg_apply")
         return y
 
     def apply_raw(self, level: int, dtype: int, x_ptr: int, y_ptr: int, stream_ptr: int) -> None:
@@ -263,6 +294,11 @@ class Mesh:
                                            ctypes.c_void_p(ev_mid), ctypes.c_void_p(ev_end)), "hyteg_p2_apply_timed")
 
 
+# hyteg_apply_batch with its arrays as addresses
+_apply_batch = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p,
+                                ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p)(("hyteg_apply_batch", C.lib))
+
+
 def apply_batch(meshes, levels, xs, ys, ieee: bool = False, stream=None):
     """ys[i] = A_i xs[i] for several (mesh, level) products in as few launches
     as possible: the 2D ones share one kernel launch per 64 meshes.  All
@@ -273,21 +309,24 @@ def apply_batch(meshes, levels, xs, ys, ieee: bool = False, stream=None):
     if n == 0:
         return ys
     dt = xs[0].dtype
+    hs, xp, yp = [], [], []
     for M, lev, x, y in zip(meshes, levels, xs, ys):
         if not (x.is_cuda and y.is_cuda) or x.dtype != dt or y.dtype != dt:
             raise ValueError("all vectors must be CUDA tensors of one dtype")
         if not (x.is_contiguous() and y.is_contiguous()):
             raise ValueError("vectors must be contiguous")
-        ns, _ = M.num_slots(lev)
+        ns = M._slots(lev)
         if x.numel() != ns or y.numel() != ns:
             raise ValueError(f"vectors of level {lev} must have {ns} elements")
+        h = M._h
+        hs.append((h.value if isinstance(h, ctypes.c_void_p) else h) or 0)
+        xp.append(x.data_ptr())
+        yp.append(y.data_ptr())
     code = Mesh._dtype_code(xs[0], ieee)
-    hs = (ctypes.c_void_p * n)(*[M._h.value if isinstance(M._h, ctypes.c_void_p) else M._h for M in meshes])
-    ls = (ctypes.c_int * n)(*levels)
-    xp = (ctypes.c_void_p * n)(*[x.data_ptr() for x in xs])
-    yp = (ctypes.c_void_p * n)(*[y.data_ptr() for y in ys])
-    C.check(C.lib.hyteg_apply_batch(hs, ls, code, xp, yp, n, ctypes.c_void_p(_stream_ptr(stream))),
-            "hyteg_apply_batch")
+    # pointer arrays as machine words: one conversion per array, not per entry
+    ah, ax, ay, al = array("Q", hs), array("Q", xp), array("Q", yp), array("i", levels)
+    C.check(_apply_batch(ah.buffer_info()[0], al.buffer_info()[0], code, ax.buffer_info()[0], ay.buffer_info()[0], n,
+                         _stream_ptr(stream)), "hyteg_apply_batch")
     return ys
 
 
