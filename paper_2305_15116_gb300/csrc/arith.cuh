@@ -116,6 +116,13 @@ __device__ __forceinline__ FF ff_split(double v) {
   return r;
 }
 
+// Whether ff_split gives v's parts (and not the NaN that marks its rows).
+__device__ __forceinline__ bool ff_in_range(double v) {
+  const unsigned mag = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
+  return mag - (unsigned(1023 + FF_EMIN) << 20) < (unsigned(FF_EMAX - FF_EMIN) << 20) ||
+         (mag | (unsigned)__double2loint(v)) == 0u;
+}
+
 // Exact float32 -> float64 of 2^-40 f with integer instructions (no
 // conversion unit): the row sums carry the weights' 2^40 scaling.  Zero
 // maps to zero; an fp32 subnormal (|f| < 2^-126, standing for less than

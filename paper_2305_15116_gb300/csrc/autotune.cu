@@ -117,8 +117,9 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
 // macros: float-float flat from 16 to 64 rows, fp32 best at 16).  On first
 // use of a level size of at least 2^20 slots the apply kernel is timed for
 // 8, 16, 32 and 64 rows (best of two launches after a warm-up) on scratch
-// vectors, per element type, and the fastest list is kept (cached per macro
-// count, level and element type for the process).  Smaller levels keep the
+// vectors, float-float and fp32, and the fastest list is kept (cached per macro
+// count, level and element type for the process); native fp64, which the direct
+// kernel takes, reports float-float's choice.  Smaller levels keep the
 // default lists (their kernels take microseconds, and the chunk already
 // shrinks until the level has 16 tiles per SM).
 cudaError_t tiles2d_autotune(Mesh& m, LevelDev& L) {
@@ -143,7 +144,7 @@ cudaError_t tiles2d_autotune(Mesh& m, LevelDev& L) {
     dev_free(m, x);
     dev_free(m, y);
   };
-  for (int dt = 1; dt <= 3 && err == cudaSuccess; ++dt) {
+  for (int dt = 1; dt <= 2 && err == cudaSuccess; ++dt) {
     const std::array<int64_t, 3> key{m.n_cells, L.n, dt};
     int best = 0;
     {
@@ -210,6 +211,7 @@ cudaError_t tiles2d_autotune(Mesh& m, LevelDev& L) {
     L.n_tiles_dt[dt] = int(tl.size());
     L.tile_rows[dt] = best;
   }
+  L.tile_rows[3] = L.tile_rows[1];
   if (err == cudaSuccess) err = dev_sync(m);
   cleanup();
   return err;

@@ -1,7 +1,7 @@
 // Native fp64 rows for the float-float kernels.
 //
 // A float-float kernel whose row read an input outside the float-float range
-// (arith.cuh) recomputes that row here, in native fp64 FMA arithmetic,
+// (arith.cuh) recomputes that row, and no other, here, in native fp64 FMA arithmetic,
 // straight from the float64 vector in global memory: the same weights (the
 // fp64 class table), the same neighbours.  Taken only for such rows, so
 // these functions favour few registers over speed.
@@ -25,6 +25,14 @@ __device__ __forceinline__ double native_row2d(const double* __restrict__ p, int
   a = __fma_rn(__ldg(w + 0), __ldg(p - len - 1), a);
   a = __fma_rn(__ldg(w + 1), __ldg(p - len), a);
   return a;
+}
+
+// Whether that row reads an input outside the float-float range (a walker
+// learns it for its whole tile only).
+__device__ __forceinline__ bool row2d_out_of_range(const double* __restrict__ p, int len) {
+  return !(ff_in_range(__ldg(p)) && ff_in_range(__ldg(p + 1)) && ff_in_range(__ldg(p - 1)) &&
+           ff_in_range(__ldg(p + len)) && ff_in_range(__ldg(p + len - 1)) && ff_in_range(__ldg(p - len - 1)) &&
+           ff_in_range(__ldg(p - len)));
 }
 
 // Slot of lattice point (x, y, z) inside a 3D macro array of level n = 2^L.

@@ -101,18 +101,18 @@ cudaError_t launch_one(const typename Body::Prm& p, int blocks, cudaStream_t s, 
 }
 
 // Launches Body over `count` meshes, blocks[i] blocks for mesh i (meshes with
-// no blocks are skipped), in launches of at most kGroupMax meshes.
-template <class Body>
+// no blocks are skipped), in launches of at most N meshes.
+template <class Body, int N = kGroupMax>
 cudaError_t launch_group(const typename Body::Prm* p, const int* blocks, int count, cudaStream_t s,
                          size_t smem = 0) {
   using Prm = typename Body::Prm;
   if (count == 1) return launch_one<Body>(p[0], blocks[0], s, smem);
   for (int i0 = 0; i0 < count;) {
-    GroupArgs<Prm, kGroupMax> g;
+    GroupArgs<Prm, N> g;
     g.count = 0;
     long long total = 0;
     int i = i0;
-    for (; i < count && g.count < kGroupMax; ++i) {
+    for (; i < count && g.count < N; ++i) {
       if (blocks[i] <= 0) continue;
       if (total + blocks[i] > 0x7FFFFFFF) break;
       g.p[g.count] = p[i];
@@ -125,7 +125,7 @@ cudaError_t launch_group(const typename Body::Prm* p, const int* blocks, int cou
     if (g.count == 0) continue;
     g.begin[g.count] = (int)total;
     const cudaError_t e =
-        launch_pdl(k_group<Body, kGroupMax>, dim3((unsigned)total), dim3(Body::kThreads), smem, s, g);
+        launch_pdl(k_group<Body, N>, dim3((unsigned)total), dim3(Body::kThreads), smem, s, g);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -24,10 +24,8 @@
 #include <type_traits>
 #include <vector>
 
-#include "arith.cuh"
+#include "direct.cuh"
 #include "fallback.cuh"
-#include "group.cuh"
-#include "hyteg_internal.h"
 
 namespace hyteg {
 
@@ -87,149 +85,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// What a launch writes at a point with (A u) = au:
-//   MODE_APPLY:    y = A u
-//   MODE_JACOBI:   y = u + omega dinv (b - A u)   (one weighted Jacobi sweep)
-//   MODE_RESIDUAL: y = b - A u
-// (u = x at the point; b and dinv in the slot layout, copies equal).
-//   MODE_PARTIAL:  y = A u inside the macros; at interface points every copy
-//                  receives its own macro's partial row instead of the sum
-constexpr int MODE_APPLY = 0, MODE_JACOBI = 1, MODE_RESIDUAL = 2, MODE_PARTIAL = 3;
-
-struct ModeArgs {
-  const void* b;
-  const void* dinv;
-  double omega;
-};
-
-// sweep modes inside the macro: u, b and dinv of the point come from the
-// staged rows
-template <int MODE, class T>
-__device__ __forceinline__ T mode_out_staged(T au, T u, T b, T d, double omega) {
-  if (MODE == MODE_APPLY) return au;
-  if (MODE == MODE_RESIDUAL) return b - au;
-  return u + (T)omega * d * (b - au);
-}
-
-template <int MODE, class T>
-__device__ __forceinline__ T mode_out(T au, const T* __restrict__ x, const ModeArgs& md, int64_t i) {
-  if (MODE == MODE_APPLY) return au;
-  const T bi = __ldg(static_cast<const T*>(md.b) + i);
-  if (MODE == MODE_RESIDUAL) return bi - au;
-  const T ui = __ldg(x + i), di = __ldg(static_cast<const T*>(md.dinv) + i);
-  return ui + (T)md.omega * di * (bi - au);
-}
-
-// ---- interface points (coarse vertices and edges), stencil mode ------------
-// Each macro holding a copy contributes its partial row (the class stencil of
-// the point in that macro: only the macro's own micro-triangles); the partials
-// are summed in ascending macro order and the sum is written to every copy.
-// Dirichlet points get y = x.  Arithmetic in the element type (fp64 for the
-// float-float apply).
-__constant__ int c_if_off[NW2][2] = {{0, -1}, {1, -1}, {-1, 0}, {0, 0}, {1, 0}, {-1, 1}, {0, 1}};
-
-__device__ __forceinline__ int64_t if_slot(int n, int x, int y) {
-  return (int64_t)y * (n + 2) - ((int64_t)y * (y + 1)) / 2 + x;
-}
-__device__ __forceinline__ double if_w(const StencilPtr& st, int64_t i, double) { return __ldg(st.d + i); }
-__device__ __forceinline__ float if_w(const StencilPtr& st, int64_t i, float) { return __ldg(st.f + i); }
-__device__ __forceinline__ double if_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float if_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-
-// The partial row of one copy of an interface point: the class stencil of
-// the point (local coordinates q) in the copy's macro.
-template <class T>
-__device__ __forceinline__ T if_partial(const T* __restrict__ x, const Inc& inc, const int q[2], int n, int64_t S,
-                                        const StencilPtr& st) {
-  const int cls = (q[0] == 0 ? 1 : 0) | (q[1] == 0 ? 2 : 0) | (q[0] + q[1] == n ? 4 : 0);
-  const int64_t base = (int64_t)inc.cell * S;
-  const int64_t wb = ((int64_t)inc.cell * NCLS2 + cls) * NW2;
-  T part = T(0);
-#pragma unroll
-  for (int k = 0; k < NW2; ++k) {
-    const int dx = c_if_off[k][0], dy = c_if_off[k][1];
-    if (((cls & 1) && dx < 0) || ((cls & 2) && dy < 0) || ((cls & 4) && dx + dy > 0)) continue;
-    part = if_fma(if_w(st, wb + k, T(0)), __ldg(x + base + if_slot(n, q[0] + dx, q[1] + dy)), part);
-  }
-  return part;
-}
-
-template <int MODE, class T>
-__device__ __forceinline__ void iface2d_point(const T* __restrict__ x, T* __restrict__ y, const Prim& p, int a,
-                                              const Inc* __restrict__ incs, int n, int64_t S, const StencilPtr& st,
-                                              const ModeArgs& md) {
-  const int wv0 = p.type == 0 ? n : n - a, wv1 = p.type == 0 ? 0 : a;  // weights on the canonical vertices
-  auto local = [&](const Inc& inc, int q[2]) {
-    q[0] = q[1] = 0;
-    if (inc.corner[0] >= 1) q[inc.corner[0] - 1] += wv0;
-    if (p.type == 1 && inc.corner[1] >= 1) q[inc.corner[1] - 1] += wv1;
-  };
-  T acc = T(0);
-  if (MODE == MODE_PARTIAL) {  // each copy keeps its own macro's partial row
-    for (int i = 0; i < p.inc_count; ++i) {
-      const Inc inc = incs[p.inc_begin + i];
-      int q[2];
-      local(inc, q);
-      y[(int64_t)inc.cell * S + if_slot(n, q[0], q[1])] = if_partial(x, inc, q, n, S, st);
-    }
-    return;
-  }
-  if (p.boundary) {
-    int q[2];
-    local(incs[p.inc_begin], q);
-    acc = __ldg(x + (int64_t)incs[p.inc_begin].cell * S + if_slot(n, q[0], q[1]));
-  } else {
-    for (int i = 0; i < p.inc_count; ++i) {
-      const Inc inc = incs[p.inc_begin + i];
-      int q[2];
-      local(inc, q);
-      acc += if_partial(x, inc, q, n, S, st);
-    }
-  }
-  if (MODE == MODE_JACOBI || MODE == MODE_RESIDUAL) {  // copies hold equal u, b and dinv: use the first
-    int q[2];
-    local(incs[p.inc_begin], q);
-    acc = mode_out<MODE>(acc, x, md, (int64_t)incs[p.inc_begin].cell * S + if_slot(n, q[0], q[1]));
-  }
-  for (int i = 0; i < p.inc_count; ++i) {
-    const Inc inc = incs[p.inc_begin + i];
-    int q[2];
-    local(inc, q);
-    y[(int64_t)inc.cell * S + if_slot(n, q[0], q[1])] = acc;
-  }
-}
-
-// A coarse vertex inside the domain (at most 32 incident macros): its copies'
-// partial rows are independent, so lane i of one warp takes copy i — walked
-// one after another by one thread, the copies' dependent loads were the
-// latency floor of the launch on small levels — and every lane adds the
-// partials in ascending copy order through shuffles, the order of the serial
-// loop, so the result is the same.
-template <int MODE, class T>
-__device__ __forceinline__ void iface2d_vertex(const T* __restrict__ x, T* __restrict__ y, const Prim& p, int lane,
-                                               const Inc* __restrict__ incs, int n, int64_t S, const StencilPtr& st,
-                                               const ModeArgs& md) {
-  const bool mine = lane < p.inc_count;
-  int q[2] = {0, 0};
-  int64_t slot = 0;
-  T part = T(0);
-  if (mine) {
-    const Inc inc = incs[p.inc_begin + lane];
-    if (inc.corner[0] >= 1) q[inc.corner[0] - 1] += n;
-    slot = (int64_t)inc.cell * S + if_slot(n, q[0], q[1]);
-    part = if_partial(x, inc, q, n, S, st);
-  }
-  if (MODE == MODE_PARTIAL) {
-    if (mine) y[slot] = part;
-    return;
-  }
-  T acc = T(0);
-  for (int i = 0; i < p.inc_count; ++i) acc += __shfl_sync(0xFFFFFFFFu, part, i);
-  if (MODE == MODE_JACOBI || MODE == MODE_RESIDUAL)  // copies hold equal u, b and dinv: use the first
-    acc = mode_out<MODE>(acc, x, md, __shfl_sync(0xFFFFFFFFu, slot, 0));
-  if (mine) y[slot] = acc;
-}
-
 // Rows in flight per warp: each lane stages its two columns of the next RING
 // rows in shared memory with cp.async, so a warp keeps RING rows outstanding
 // without holding them in registers.
@@ -237,9 +92,9 @@ constexpr int RING = 3;  // rows in flight; the walk is unrolled by three
 constexpr int THREADS2D = 256;
 
 // One launch does the whole apply: blocks 0 .. n_if_blocks-1 take the
-// interface items (two items of up to 128 points per block), the others the
-// macro-interior tiles.  The two parts write disjoint slots and read only x,
-// so they run side by side.
+// interface items (one per warp, lattice.cuh; arithmetic in the element type,
+// fp64 for the float-float apply), the others the macro-interior tiles.  The
+// two parts write disjoint slots and read only x, so they run side by side.
 // Threads per block (the sweep modes stage rows of b beside x; the inverse
 // diagonal of a macro-interior point is the macro's constant 1 / centre
 // weight, so it is not read).
@@ -254,8 +109,8 @@ template <class P, int MODE>
 __device__ __forceinline__ void apply2d_block(int block, const typename P::T* __restrict__ x,
                                               typename P::T* __restrict__ y, const int4* __restrict__ tiles,
                                               int n_tiles, int64_t n_warps, int64_t S, int n, const StencilPtr& st,
-                                              const int4* __restrict__ items, int n_items,
-                                              const Prim* __restrict__ prims, const Inc* __restrict__ incs,
+                                              const IfItem* __restrict__ items, int n_items,
+                                              const Inc* __restrict__ incs,
                                               int n_if_blocks, const ModeArgs& md,
                                               typename P::T (*ring_all)[RING][32][2],
                                               typename P::T (*ringb_all)[RING][32][2]) {
@@ -264,18 +119,11 @@ __device__ __forceinline__ void apply2d_block(int block, const typename P::T* __
   constexpr bool SWEEP = MODE == MODE_JACOBI || MODE == MODE_RESIDUAL;
   static_assert(!SWEEP || sizeof(T) == 4, "the sweep modes are built for fp32");
   if (block < n_if_blocks) {
-    const int item = (THR / 128) * block + (int)(threadIdx.x >> 7);
+    const int item = (THR / 32) * block + (int)(threadIdx.x >> 5);
     if (item >= n_items) return;
-    const int4 it = items[item];
-    const int t = (int)(threadIdx.x & 127);
-    const Prim p = prims[it.x];
+    const IfItem it = items[item];
     pdl_wait();  // the vectors after the previous kernel in the stream (group.cuh)
-    if (p.type == 0 && !p.boundary && p.inc_count <= 32) {
-      if (t < 32) iface2d_vertex<MODE, T>(x, y, p, t, incs, n, S, st, md);  // the item's first warp
-      return;
-    }
-    const int a = it.z + t;
-    if (a < it.w) iface2d_point<MODE, T>(x, y, p, a, incs, n, S, st, md);
+    apply_item<2, MODE, false, false, T>(x, y, it, (int)(threadIdx.x & 31), incs, n, S, st, md);
     return;
   }
   const int64_t warp = ((int64_t)(block - n_if_blocks) * blockDim.x + threadIdx.x) >> 5;
@@ -457,15 +305,18 @@ __device__ __forceinline__ void apply2d_block(int block, const typename P::T* __
   }
   cp_async_wait<0>();
   if constexpr (P::kPoison) {
-    // a row of this lane read an input outside the float-float range: its
-    // two columns of the tile again, in native fp64 from memory
+    // a row of this lane read an input outside the float-float range: those of
+    // its two columns of the tile again, in native fp64 from memory
     if (P::marked(mk)) {
       const double* wd = st.d + wb;
       Cursor rw;
       rw.init(n, t.y);
       for (int r = t.y; r < t.z; ++r) {
-        if (wa && ca < rw.len - 1) ym[rw.off + ca] = native_row2d(xm + rw.off + ca, rw.len, wd);
-        if (wbb && cb < rw.len - 1) ym[rw.off + cb] = native_row2d(xm + rw.off + cb, rw.len, wd);
+        const double* const xr = xm + rw.off;
+        if (wa && ca < rw.len - 1 && row2d_out_of_range(xr + ca, rw.len))
+          ym[rw.off + ca] = native_row2d(xr + ca, rw.len, wd);
+        if (wbb && cb < rw.len - 1 && row2d_out_of_range(xr + cb, rw.len))
+          ym[rw.off + cb] = native_row2d(xr + cb, rw.len, wd);
         rw.next();
       }
     }
@@ -484,8 +335,7 @@ __global__ void __launch_bounds__(Thr2<MODE>::value, MinBlocks2<P>::value) k_int
                                                           typename P::T* __restrict__ y,
                                                           const int4* __restrict__ tiles, int n_tiles,
                                                           int64_t n_warps, int64_t S, int n, StencilPtr st,
-                                                          const int4* __restrict__ items, int n_items,
-                                                          const Prim* __restrict__ prims,
+                                                          const IfItem* __restrict__ items, int n_items,
                                                           const Inc* __restrict__ incs, int n_if_blocks,
                                                           ModeArgs md) {
   using T = typename P::T;
@@ -494,7 +344,7 @@ __global__ void __launch_bounds__(Thr2<MODE>::value, MinBlocks2<P>::value) k_int
   __shared__ __align__(8) T ring_all[THR / 32][RING][32][2];
   __shared__ __align__(8) T ringb_all[SWEEP ? THR / 32 : 1][RING][32][2];
   pdl_trigger();
-  apply2d_block<P, MODE>((int)blockIdx.x, x, y, tiles, n_tiles, n_warps, S, n, st, items, n_items, prims, incs,
+  apply2d_block<P, MODE>((int)blockIdx.x, x, y, tiles, n_tiles, n_warps, S, n, st, items, n_items, incs,
                          n_if_blocks, md, ring_all, ringb_all);
 }
 
@@ -507,8 +357,7 @@ struct Apply2dDesc {
   const void* x;
   void* y;
   const int4* tiles;
-  const int4* items;
-  const Prim* prims;
+  const IfItem* items;
   const Inc* incs;
   StencilPtr st;
   ModeArgs md;  // the sweep modes' b, inverse diagonal and omega
@@ -541,8 +390,96 @@ __global__ void __launch_bounds__(Thr2<MODE>::value, MinBlocks2<P>::value) k_int
   }
   const Apply2dDesc& d = b.d[lo];
   apply2d_block<P, MODE>((int)blockIdx.x - d.block_begin, static_cast<const T*>(d.x), static_cast<T*>(d.y), d.tiles,
-                         d.n_tiles > 0 ? d.n_tiles : 1, d.n_warps, d.S, d.n, d.st, d.items, d.n_items, d.prims,
+                         d.n_tiles > 0 ? d.n_tiles : 1, d.n_warps, d.S, d.n, d.st, d.items, d.n_items,
                          d.incs, d.n_if_blocks, d.md, ring_all, ringb_all);
+}
+
+// ---- small vectors: one thread per macro-interior point -----------------------------
+// A walk's time on a small level is its chain of rows (each step waits for a
+// copy, 8 rows at least), 8 us for a product of a few us of latency and work.
+// In the direct form every neighbour is loaded at once.
+template <class P, int MODE>
+struct Direct2 {
+  using T = typename P::T;
+  static constexpr int kThreads = 256;
+  static constexpr bool kLateWait = true;  // the tables first
+  struct Prm {
+    const T* x;
+    T* y;
+    const IfItem* items;
+    const Inc* incs;
+    StencilPtr st;
+    ModeArgs md;
+    int64_t S;
+    int n, n_pts, bpm, n_items, n_if_blocks;  // per macro: interior points, blocks
+  };
+  static __device__ __forceinline__ void run(const Prm& p, int block, int) {
+    if (block < p.n_if_blocks) {
+      const int item = (kThreads / 32) * block + (int)(threadIdx.x >> 5);
+      if (item >= p.n_items) return;
+      const IfItem it = p.items[item];
+      pdl_wait();
+      apply_item<2, MODE, false, false, T>(p.x, p.y, it, (int)(threadIdx.x & 31), p.incs, p.n, p.S, p.st, p.md);
+      return;
+    }
+    const int b = block - p.n_if_blocks;
+    const int m = b / p.bpm;
+    const int t = (b - m * p.bpm) * kThreads + (int)threadIdx.x;
+    if (t >= p.n_pts) return;
+    int slot, A;
+    inner_point2(t, p.n, slot, A);
+    const int64_t wb = (int64_t)m * (NCLS2 * NW2);
+    InnerW<2, P> W;
+    W.load(p.st, wb);
+    const int64_t i = (int64_t)m * p.S + slot;
+    T bi = T(0), di = T(0), uc;
+    if (MODE == MODE_JACOBI) di = __ldg(static_cast<const T*>(p.md.dinv) + i);
+    pdl_wait();
+    if (MODE == MODE_JACOBI || MODE == MODE_RESIDUAL) bi = ld<false>(static_cast<const T*>(p.md.b) + i);
+    const T r = inner_row<2, P, false>(p.x + i, Off7(0, A), W, p.st, wb, uc);
+    p.y[i] = mode_out_staged<MODE, T>(r, uc, bi, di, p.md.omega);
+  }
+};
+
+template <class P, int MODE>
+cudaError_t launch_direct(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
+                          const ModeArgs* md, int count, cudaStream_t s) {
+  using B = Direct2<P, MODE>;
+  using T = typename P::T;
+  std::vector<typename B::Prm> prm(count);
+  std::vector<int> blocks(count);
+  for (int i = 0; i < count; ++i) {
+    const Mesh& m = *ms[i];
+    const LevelDev& L = m.levels[levels[i]];
+    typename B::Prm& p = prm[i];
+    p.x = static_cast<const T*>(xs[i]);
+    p.y = static_cast<T*>(ys[i]);
+    p.items = L.ifi;
+    p.incs = m.d_incs;
+    p.st = StencilPtr{L.st64, L.st32, L.st_hi, L.st_lo};
+    p.md = md ? md[i] : ModeArgs{nullptr, nullptr, 0.0};
+    p.S = L.slots_per_macro;
+    p.n = L.n;
+    p.n_pts = L.n > 2 ? (L.n - 1) * (L.n - 2) / 2 : 0;
+    p.bpm = (p.n_pts + B::kThreads - 1) / B::kThreads;
+    p.n_items = L.n_ifi;
+    p.n_if_blocks = (L.n_ifi + B::kThreads / 32 - 1) / (B::kThreads / 32);
+    blocks[i] = p.n_if_blocks + p.bpm * int(m.n_cells);
+  }
+  return launch_group<B, BATCH2D>(prm.data(), blocks.data(), count, s);
+}
+
+// Whether a level's products and sweeps take the direct kernel: small vectors
+// (us per apply, direct / walker, float64: 268k slots 6.0 / 9.1, 1.0M slots 16.2
+// / 9.2; fp32 alike up to 0.3M slots, 1.0M 5.2 / 4.4; a V-cycle on 32
+// macro-triangles at level 10 679 / 692), and native fp64 at any size, which the
+// fp64 pipe bounds and the occupancy of single points suits (17k slots 4.3 / 9.3,
+// 4.0M slots 51 / 65, 67M slots 842 / 896: 7 operations per point at 94 % of
+// the nominal fp64 rate).  Both forms round alike, and recompute the same rows
+// in native fp64, so a result does not depend on the choice.
+template <class P>
+bool takes_direct(const Mesh& m, const LevelDev& L) {
+  return std::is_same<P, ArF64Native>::value || L.slots_per_macro * m.n_cells <= kDirect2MaxSlots;
 }
 
 // Element-type index of a policy (1 float-float, 2 fp32, 3 native fp64).
@@ -572,64 +509,94 @@ cudaError_t launch_on(const Mesh& m, const LevelDev& L, const int4* tiles, int n
   const int64_t n_warps = (int64_t)n_tiles * m.n_cells;
   const int threads = Thr2<MODE>::value;
   const int64_t int_blocks = (n_warps * 32 + threads - 1) / threads;
-  const int per = threads / 128;  // interface items per block
-  const int if_blocks = (L.n_items + per - 1) / per;
+  const int per = threads / 32;  // interface items per block
+  const int if_blocks = (L.n_ifi + per - 1) / per;
   if (int_blocks + if_blocks == 0) return cudaSuccess;
   StencilPtr st{L.st64, L.st32, L.st_hi, L.st_lo};
   return launch_pdl(k_interior2d<P, MODE>, dim3((unsigned)(int_blocks + if_blocks)), dim3(threads), 0, s,
                     (const typename P::T*)x, (typename P::T*)y, tiles, n_tiles > 0 ? n_tiles : 1, n_warps,
-                    L.slots_per_macro, L.n, st, (const int4*)L.items, L.n_items, (const Prim*)m.d_prims,
-                    (const Inc*)m.d_incs, if_blocks, md);
+                    L.slots_per_macro, L.n, st, (const IfItem*)L.ifi, L.n_ifi, (const Inc*)m.d_incs, if_blocks, md);
 }
 
 template <class P, int MODE>
 cudaError_t launch(const Mesh& m, const LevelDev& L, const void* x, void* y, cudaStream_t s, const ModeArgs& md) {
-  const int4* tiles = nullptr;
-  int n_tiles = 0;
-  tiles_of<P>(L, &tiles, &n_tiles);
-  return launch_on<P, MODE>(m, L, tiles, n_tiles, x, y, s, md);
+  if (takes_direct<P>(m, L)) {
+    const Mesh* mp = &m;
+    return launch_direct<P, MODE>(&mp, &L.level, &x, &y, &md, 1, s);
+  }
+  if constexpr (!std::is_same<P, ArF64Native>::value) {
+    const int4* tiles = nullptr;
+    int n_tiles = 0;
+    tiles_of<P>(L, &tiles, &n_tiles);
+    return launch_on<P, MODE>(m, L, tiles, n_tiles, x, y, s, md);
+  }
+  return cudaErrorInvalidValue;
 }
 
 template <class P, int MODE = MODE_APPLY>
 cudaError_t launch_batch_t(const Mesh* const* meshes, const int* levels, const void* const* xs, void* const* ys,
                            int count, cudaStream_t s, const ModeArgs* mds = nullptr) {
   constexpr int THR = Thr2<MODE>::value;
-  Apply2dBatch b;
-  for (int i0 = 0; i0 < count; i0 += BATCH2D) {
-    b.count = 0;
-    int blocks = 0;
-    for (int i = i0; i < count && i < i0 + BATCH2D; ++i) {
-      const Mesh& m = *meshes[i];
-      const LevelDev& L = m.levels[levels[i]];
-      const int4* tiles = nullptr;
-      int n_tiles = 0;
-      tiles_of<P>(L, &tiles, &n_tiles);
-      const int64_t n_warps = (int64_t)n_tiles * m.n_cells;
-      const int64_t int_blocks = (n_warps * 32 + THR - 1) / THR;
-      const int if_blocks = (L.n_items + THR / 128 - 1) / (THR / 128);
-      if (int_blocks + if_blocks == 0) continue;
-      if ((int64_t)blocks + int_blocks + if_blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-      Apply2dDesc& d = b.d[b.count++];
-      d.x = xs[i];
-      d.y = ys[i];
-      d.tiles = tiles;
-      d.items = L.items;
-      d.prims = m.d_prims;
-      d.incs = m.d_incs;
-      d.st = StencilPtr{L.st64, L.st32, L.st_hi, L.st_lo};
-      d.md = mds ? mds[i] : ModeArgs{nullptr, nullptr, 0.0};
-      d.n_warps = n_warps;
-      d.S = L.slots_per_macro;
-      d.n_tiles = n_tiles;
-      d.n = L.n;
-      d.n_items = L.n_items;
-      d.n_if_blocks = if_blocks;
-      d.block_begin = blocks;
-      blocks += int(int_blocks + if_blocks);
+  // small ones directly, in launches of their own
+  std::vector<int> small, large;
+  for (int i = 0; i < count; ++i)
+    (takes_direct<P>(*meshes[i], meshes[i]->levels[levels[i]]) ? small : large).push_back(i);
+  if (!small.empty()) {
+    std::vector<const Mesh*> mm;
+    std::vector<int> lv;
+    std::vector<const void*> xx;
+    std::vector<void*> yy;
+    std::vector<ModeArgs> mo;
+    for (int i : small) {
+      mm.push_back(meshes[i]);
+      lv.push_back(levels[i]);
+      xx.push_back(xs[i]);
+      yy.push_back(ys[i]);
+      if (mds) mo.push_back(mds[i]);
     }
-    if (b.count == 0) continue;
-    const cudaError_t e = launch_pdl(k_interior2d_batch<P, MODE>, dim3(blocks), dim3(THR), 0, s, b);
+    const cudaError_t e = launch_direct<P, MODE>(mm.data(), lv.data(), xx.data(), yy.data(),
+                                                 mds ? mo.data() : nullptr, int(mm.size()), s);
     if (e != cudaSuccess) return e;
+  }
+  if constexpr (!std::is_same<P, ArF64Native>::value) {
+    Apply2dBatch b;
+    const int n_large = int(large.size());
+    for (int i0 = 0; i0 < n_large; i0 += BATCH2D) {
+      b.count = 0;
+      int blocks = 0;
+      for (int j = i0; j < n_large && j < i0 + BATCH2D; ++j) {
+        const int i = large[j];
+        const Mesh& m = *meshes[i];
+        const LevelDev& L = m.levels[levels[i]];
+        const int4* tiles = nullptr;
+        int n_tiles = 0;
+        tiles_of<P>(L, &tiles, &n_tiles);
+        const int64_t n_warps = (int64_t)n_tiles * m.n_cells;
+        const int64_t int_blocks = (n_warps * 32 + THR - 1) / THR;
+        const int if_blocks = (L.n_ifi + THR / 32 - 1) / (THR / 32);
+        if (int_blocks + if_blocks == 0) continue;
+        if ((int64_t)blocks + int_blocks + if_blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+        Apply2dDesc& d = b.d[b.count++];
+        d.x = xs[i];
+        d.y = ys[i];
+        d.tiles = tiles;
+        d.items = L.ifi;
+        d.incs = m.d_incs;
+        d.st = StencilPtr{L.st64, L.st32, L.st_hi, L.st_lo};
+        d.md = mds ? mds[i] : ModeArgs{nullptr, nullptr, 0.0};
+        d.n_warps = n_warps;
+        d.S = L.slots_per_macro;
+        d.n_tiles = n_tiles;
+        d.n = L.n;
+        d.n_items = L.n_ifi;
+        d.n_if_blocks = if_blocks;
+        d.block_begin = blocks;
+        blocks += int(int_blocks + if_blocks);
+      }
+      if (b.count == 0) continue;
+      const cudaError_t e = launch_pdl(k_interior2d_batch<P, MODE>, dim3(blocks), dim3(THR), 0, s, b);
+      if (e != cudaSuccess) return e;
+    }
   }
   return cudaSuccess;
 }
@@ -663,7 +630,6 @@ cudaError_t launch_apply2d_tiles(int dtype, const Mesh& m, const LevelDev& L, co
   switch (dtype) {
     case 1: return launch_on<ArF64FF, MODE_APPLY>(m, L, tiles, n_tiles, x, y, s, md);
     case 2: return launch_on<ArF32, MODE_APPLY>(m, L, tiles, n_tiles, x, y, s, md);
-    case 3: return launch_on<ArF64Native, MODE_APPLY>(m, L, tiles, n_tiles, x, y, s, md);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -399,8 +399,10 @@ struct March3 {
         if constexpr (P::kPoison) {
           if (mine && P::bad(acc)) {  // an input outside the float-float range: native fp64 rows
             const int z = s - 1, px = k - (q - k * (k + 1) / 2), py = n - z - k;
-            ra = march_native_row(xa, n, px, py, z, p.st.d + wa);
-            rb = march_native_row(xb, n, px, py, z, p.st.d + wb);
+            float sa, sb;
+            f2_unpack(acc.s, sa, sb);
+            if (sa != sa) ra = march_native_row(xa, n, px, py, z, p.st.d + wa);
+            if (sb != sb) rb = march_native_row(xb, n, px, py, z, p.st.d + wb);
           }
         }
         if constexpr (kSweep) {
