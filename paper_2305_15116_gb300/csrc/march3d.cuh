@@ -177,7 +177,9 @@ struct March3 {
   static constexpr int kPlanes = kSplit ? (STRIDE <= 512 ? 4 : 3) : 0;
   static constexpr bool kReread = kPlanes == 4;
   static constexpr int kDepth = kReread ? 4 : sizeof(T) == 4 && STRIDE <= 512 ? 6 : 3;
-  static constexpr int kMinBlocks = STRIDE > 512 ? 1 : sizeof(T) == 4 ? 4 : 2;
+  // fp32: three blocks per SM.  At four the 64 registers spill around the
+  // interface step and in the marching (level 7, 72 macro-tets: 105 against 94 us).
+  static constexpr int kMinBlocks = STRIDE > 512 ? 1 : sizeof(T) == 4 ? 3 : 2;
   static constexpr int kRounds = (STRIDE + MARCH_COLS - 1) / MARCH_COLS;
   static constexpr bool kSweep = MODE == MODE_JACOBI || MODE == MODE_RESIDUAL;
   struct Prm {
@@ -280,30 +282,27 @@ struct March3 {
     const int64_t N1 = n + 1, B1 = N1 - s0;
     const int c0 = count(s0);
     const int E0 = (int)((N1 * (N1 + 1) * (N1 + 2) - B1 * (B1 + 1) * (B1 + 2)) / 6) + c0 - 1;
-    // the elements this thread stages (and splits): e with e > qmax - c(z),
-    // beyond the block's last one never
-    int el[kRounds];
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int e = tid + r * MARCH_COLS;
-      el[r] = e <= qmax - max(qmin, 0) ? e - qmax : -0x40000000;
-    }
+    // The elements e = tid + r MARCH_COLS, qmax - c(z) < e <= emax, are staged
+    // (and split) by this thread: one bound for the tests of all of them, and
+    // the second macro's addresses as an offset, which kept 18 registers free.
+    const int emax = qmax - max(qmin, 0);
+    const int below = emax - tid;
+    auto staged = [&](int r, int cz) { return (unsigned)(below - r * MARCH_COLS) < (unsigned)max(cz + emax - qmax, 0); };
+    const int pair_off = two ? (int)p.S : 0;
     int z_st = s0, c_st = c0;  // the next slice to stage
     const T* ga = xa + (E0 - qmax + tid);
-    const T* gb = xb + (E0 - qmax + tid);
     auto stage = [&](auto slot_c) {
       constexpr int at = decltype(slot_c)::value % kDepth * 2 * STRIDE;
       if (z_st <= s1) {
 #pragma unroll
         for (int r = 0; r < kRounds; ++r)
-          if (el[r] + c_st > 0) {
+          if (staged(r, c_st)) {
             cp_async_one(ring + at + tid + r * MARCH_COLS, ga + r * MARCH_COLS);
-            cp_async_one(ring + at + STRIDE + tid + r * MARCH_COLS, gb + r * MARCH_COLS);
+            cp_async_one(ring + at + STRIDE + tid + r * MARCH_COLS, ga + pair_off + r * MARCH_COLS);
           }
         ++z_st;
         c_st -= n + 2 - z_st;  // c(z) - c(z+1) = n+1-z
         ga += c_st;
-        gb += c_st;
       }
       cp_async_commit();
     };
@@ -322,7 +321,7 @@ struct March3 {
         }
 #pragma unroll
         for (int r = 0; r < kRounds; ++r)
-          if (el[r] + c_sp > 0) {
+          if (staged(r, c_sp)) {
             const FF a = ff_split(va[r]), b = ff_split(vb[r]);
             planes[pl + tid + r * MARCH_COLS] = make_ulonglong2(f2_pack(a.h, b.h), f2_pack(a.l, b.l));
           }
@@ -334,13 +333,11 @@ struct March3 {
     const int c = qmax - q;  // this column's element
     const int cp = c + A, cm = c - A;
     T* ya = p.y + (int64_t)m0 * p.S + (E0 - c0 - q);  // at the point of slice s-1
-    T* yb = p.y + (int64_t)m1 * p.S + (E0 - c0 - q);
     int c_now = c0;
-    const T *bpa = nullptr, *bpb = nullptr;  // sweep modes: b at the point of slice s
+    const T* bp = nullptr;  // sweep modes: b at the point of slice s
     T ba = T(0), bb = T(0), da = T(0), db = T(0);
     if (kSweep) {
-      bpa = static_cast<const T*>(p.md.b) + (int64_t)m0 * p.S + (E0 - q);
-      bpb = static_cast<const T*>(p.md.b) + (int64_t)m1 * p.S + (E0 - q);
+      bp = static_cast<const T*>(p.md.b) + (int64_t)m0 * p.S + (E0 - q);
     }
     if (MODE == MODE_JACOBI && zhi >= zlo) {  // the inverse diagonal is one value inside a macro
       const T* dv = static_cast<const T*>(p.md.dinv);
@@ -413,23 +410,21 @@ struct March3 {
         }
         if (mine) {
           *ya = ra;
-          if (two) *yb = rb;
+          if (pair_off) ya[pair_off] = rb;
         }
       }
       if constexpr (kSweep) {
         if (s >= zlo && s <= zhi) {
-          ba = ld<false>(bpa);
-          bb = ld<false>(bpb);
+          ba = ld<false>(bp);
+          bb = ld<false>(bp + pair_off);
         }
-        bpa += c_now - (n + 1 - s);
-        bpb += c_now - (n + 1 - s);
+        bp += c_now - (n + 1 - s);
       }
       Q::first(acc, W(0), now.c);
       Q::sym(acc, W(1), vm, now.p1);
       Q::sym(acc, W(2), l0, now.A1);
       Q::sym(acc, W(3), now.A0, l1);
       ya += c_now;
-      yb += c_now;
       c_now -= n + 1 - s;
     };
 
