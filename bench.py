@@ -169,9 +169,9 @@ def setup(name, device, dtype_code, level=None):
     interior = coarse.n_cells * ((n - 1) * (n - 2) // 2 if coarse.dim == 2 else (n - 1) * (n - 2) * (n - 3) // 6)
     slab = True  # every apply kernel writes every slot (interface copies included)
     # the library's kernel launches per apply: 2D one (macro interiors and
-    # interface points together), 3D one likewise; P2 the row and boundary
-    # kernels and the vertex and edge reductions
-    launches = 4 if p2 else 1
+    # interface points together), 3D one likewise; P2 one for the rows and
+    # boundary points and one for the vertex and edge reductions
+    launches = 2 if p2 else 1
     if p2:
         kernel = "k_p2_apply"
         raw = lambda l, c, xp, yp, sp: M.p2_apply_timed(l, c, xp, yp, sp, 0, 0, 0)

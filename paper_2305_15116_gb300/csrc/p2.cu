@@ -18,6 +18,7 @@
 
 #include "arith.cuh"
 #include "fallback.cuh"
+#include "group.cuh"
 #include "hyteg_internal.h"
 
 namespace hyteg {
@@ -89,11 +90,8 @@ __device__ __forceinline__ typename P::T row(const typename P::T* __restrict__ x
 // (x = 0..n), column x = 0 (y = 1..n), the long edge x + y = n (x = 1..n-1)
 // and the line x + y = n-1 (x = 1..n-2).
 template <class P>
-__global__ void __launch_bounds__(128) k_p2_boundary(const typename P::T* __restrict__ x,
-                                                     typename P::T* __restrict__ y, Geo G, StencilPtr st,
-                                                     int n_points) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_points) return;
+__device__ __forceinline__ void p2_boundary_point(const typename P::T* __restrict__ x, typename P::T* __restrict__ y,
+                                                  const Geo& G, const StencilPtr& st, int64_t cell, int i) {
   const int n = G.n;
   int px, py;
   if (i <= n) {
@@ -105,7 +103,6 @@ __global__ void __launch_bounds__(128) k_p2_boundary(const typename P::T* __rest
   } else {
     px = i - 3 * n + 1, py = n - 1 - px;
   }
-  const int64_t cell = blockIdx.y;
   const typename P::T* __restrict__ xm = x + cell * G.S2;
   typename P::T* __restrict__ ym = y + cell * G.S2;
   const int64_t wb = cell * P2W;
@@ -130,7 +127,7 @@ __global__ void __launch_bounds__(128) k_p2_boundary(const typename P::T* __rest
 // whose class is interior:
 //   V(x,y): x >= 1, y >= 1, x + y <= n-1     X(x,y): y >= 1, x + y <= n-1
 //   Y(x,y): x >= 1, x + y <= n-1              XY(x,y): x + y <= n-2
-// The DoFs on the macro's edges (their partial rows) come from k_p2_boundary.
+// The DoFs on the macro's edges (their partial rows) come from p2_boundary_point.
 // For the Laplacian the coupling of a vertex with the edge opposite to it in
 // a triangle vanishes: integral of (4 lambda_i - 1) lambda_k is
 // 4|T|/12 - |T|/3 = 0.  The host sets those weights to zero (6 of the 12 edge
@@ -216,17 +213,28 @@ struct P2Ring {
 };
 constexpr int P2THREADS = 256;
 
+// The first blocks (per_cell for each macro) are p2_boundary_point's work.  A
+// macro's boundary points are few and wait on their gathers; beside the rows
+// that costs nothing.  Four launches as two (with k_p2_reduce): 421 -> 405 us
+// at level 10 with 32 macros (fp32 150 -> 135), 45 -> 26 us at level 7 with 24.
 template <class P>
 __global__ void __launch_bounds__(P2THREADS) k_p2_rows(const typename P::T* __restrict__ x, typename P::T* __restrict__ y,
                                                        const int4* __restrict__ tiles, int n_tiles, int64_t n_warps,
-                                                       Geo G, StencilPtr st) {
+                                                       Geo G, StencilPtr st, int n_points, int per_cell,
+                                                       int n_boundary) {
+  pdl_trigger();
+  if ((int)blockIdx.x < n_boundary) {
+    const int cell = blockIdx.x / per_cell, i = (blockIdx.x - cell * per_cell) * P2THREADS + threadIdx.x;
+    if (i < n_points) p2_boundary_point<P>(x, y, G, st, cell, i);
+    return;
+  }
   using T = typename P::T;
   using V = typename P::V;
   constexpr bool REG = false;  // weights from shared memory: fewer registers, more resident warps
   constexpr int P2RING = P2Ring<T>::value;
   __shared__ T ring_all[P2THREADS / 32][P2RING][4][32];
   __shared__ typename P::W wslice_all[P2THREADS / 32][REG ? 1 : 46];
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t warp = ((int64_t)(blockIdx.x - n_boundary) * P2THREADS + threadIdx.x) >> 5;
   if (warp >= n_warps) return;  // whole warps leave together
   const int lane = threadIdx.x & 31;
   const int wid = threadIdx.x >> 5;
@@ -419,10 +427,9 @@ __global__ void __launch_bounds__(P2THREADS) k_p2_rows(const typename P::T* __re
 // Edge DoFs on coarse edges: sum the copies' partial rows in ascending macro
 // order and write the sum to every copy (Dirichlet edges: y = x).
 template <class T>
-__global__ void __launch_bounds__(128) k_p2_edge_reduce(const T* __restrict__ x, T* __restrict__ y,
-                                                        const int4* __restrict__ items, const Prim* __restrict__ prims,
-                                                        const Inc* __restrict__ incs, Geo G) {
-  const int4 it = items[blockIdx.x];
+__device__ __forceinline__ void p2_edge_reduce(const T* __restrict__ x, T* __restrict__ y, const int4& it,
+                                                const Prim* __restrict__ prims, const Inc* __restrict__ incs,
+                                                const Geo& G) {
   const int t = it.y + threadIdx.x;
   if (t >= it.z) return;
   const Prim p = prims[it.x];
@@ -456,10 +463,9 @@ __global__ void __launch_bounds__(128) k_p2_edge_reduce(const T* __restrict__ x,
 // Vertex DoFs on coarse vertices and edges: as the P1 reduction, in the P2
 // macro blocks.
 template <class T>
-__global__ void __launch_bounds__(128) k_p2_vertex_reduce(const T* __restrict__ x, T* __restrict__ y,
-                                                          const int4* __restrict__ items, const Prim* __restrict__ prims,
-                                                          const Inc* __restrict__ incs, Geo G) {
-  const int4 it = items[blockIdx.x];
+__device__ __forceinline__ void p2_vertex_reduce(const T* __restrict__ x, T* __restrict__ y, const int4& it,
+                                                const Prim* __restrict__ prims, const Inc* __restrict__ incs,
+                                                const Geo& G) {
   const int a = it.z + threadIdx.x;
   if (a >= it.w) return;
   const Prim p = prims[it.x];
@@ -488,6 +494,21 @@ __global__ void __launch_bounds__(128) k_p2_vertex_reduce(const T* __restrict__ 
   for (int i = 0; i < p.inc_count; ++i) y[slot_of(i)] = acc;
 }
 
+// Both reductions in one launch, which is placed while the row kernel drains.
+template <class T>
+__global__ void __launch_bounds__(128) k_p2_reduce(const T* __restrict__ x, T* __restrict__ y,
+                                                   const int4* __restrict__ v_items, int n_v,
+                                                   const int4* __restrict__ e_items, const Prim* __restrict__ prims,
+                                                   const Inc* __restrict__ incs, Geo G) {
+  const int b = (int)blockIdx.x;
+  const int4 it = b < n_v ? v_items[b] : e_items[b - n_v];
+  pdl_wait();
+  if (b < n_v)
+    p2_vertex_reduce<T>(x, y, it, prims, incs, G);
+  else
+    p2_edge_reduce<T>(x, y, it, prims, incs, G);
+}
+
 template <class P>
 cudaError_t launch_t(const Mesh& m, const LevelDev& L, const void* x, void* y, cudaStream_t s, cudaEvent_t ev_mid,
                      const char** what) {
@@ -499,25 +520,22 @@ cudaError_t launch_t(const Mesh& m, const LevelDev& L, const void* x, void* y, c
   G.S2 = G.Sv + 3 * G.Se;
   StencilPtr st{L.p2_st64, L.p2_st32, L.p2_hi, L.p2_lo};
   *what = "P2 row kernel";
-  cudaError_t e = cudaSuccess;
-  if (L.n_p2_tiles > 0) {
-    const int64_t n_warps = (int64_t)L.n_p2_tiles * m.n_cells;
-    const int64_t blocks = (n_warps * 32 + P2THREADS - 1) / P2THREADS;
-    k_p2_rows<P><<<(unsigned)blocks, P2THREADS, 0, s>>>((const T*)x, (T*)y, L.p2_tiles, L.n_p2_tiles, n_warps, G, st);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  *what = "P2 boundary kernel";
-  const int nb = L.n == 1 ? 3 : 4 * L.n - 2;
-  k_p2_boundary<P><<<dim3((unsigned)((nb + 127) / 128), (unsigned)m.n_cells), 128, 0, s>>>((const T*)x, (T*)y, G, st,
-                                                                                             nb);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const int64_t n_warps = (int64_t)L.n_p2_tiles * m.n_cells;
+  const int nb = L.n == 1 ? 3 : 4 * L.n - 2, per_cell = (nb + P2THREADS - 1) / P2THREADS;
+  const int64_t n_boundary = (int64_t)per_cell * m.n_cells;
+  const int64_t blocks = n_boundary + (n_warps * 32 + P2THREADS - 1) / P2THREADS;
+  if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  k_p2_rows<P><<<(unsigned)blocks, P2THREADS, 0, s>>>((const T*)x, (T*)y, L.p2_tiles, L.n_p2_tiles, n_warps, G, st, nb,
+                                                      per_cell, (int)n_boundary);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   if (ev_mid && (e = cudaEventRecord(ev_mid, s)) != cudaSuccess) return e;
   *what = "P2 interface kernels";
-  if (L.n_items > 0)
-    k_p2_vertex_reduce<T><<<L.n_items, 128, 0, s>>>((const T*)x, (T*)y, L.items, m.d_prims, m.d_incs, G);
-  if (L.n_p2_items > 0)
-    k_p2_edge_reduce<T><<<L.n_p2_items, 128, 0, s>>>((const T*)x, (T*)y, L.p2_items, m.d_prims, m.d_incs, G);
-  return cudaGetLastError();
+  const int n_reduce = L.n_items + L.n_p2_items;
+  if (n_reduce > 0)
+    return launch_pdl(k_p2_reduce<T>, dim3((unsigned)n_reduce), dim3(128), 0, s, (const T*)x, (T*)y, L.items,
+                      L.n_items, L.p2_items, m.d_prims, m.d_incs, G);
+  return cudaSuccess;
 }
 
 }  // namespace
