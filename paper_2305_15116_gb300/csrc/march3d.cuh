@@ -21,11 +21,11 @@
 // Measured (us per apply, this kernel with its interface step / the kernels
 // before it, which decoded each slice's points by index with 15 shared loads
 // each, or above n = 64 walked along rows, and summed the interface in a launch
-// of their own): level 6, 384 macro-tets float-float 236 / 298, fp32 80 / 131;
-// level 7, 72 macro-tets 271 / 572, 90 / 243.  Executed instructions per slot:
+// of their own): level 6, 384 macro-tets float-float 235 / 298, fp32 86 / 131;
+// level 7, 72 macro-tets 269 / 572, 94 / 244.  Executed instructions per slot:
 // float-float 331 -> 160, fp32 181 -> 54 (level 7); without the interface step
 // 157 and 47 us at level 6.  What bounds it: latency between the barriers with 16 warps per SM
-// (issue 46 %, fp32 pipe 40 %, shared-memory wavefronts 55 % in float-float;
+// in float-float, 24 in fp32 (issue 40 / 50 %, L1 and shared memory 55 / 63 %;
 // more blocks per SM with fewer registers ran slower), and the interface
 // points' gathers, whose rows lie a slice apart.
 //
