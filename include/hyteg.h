@@ -113,7 +113,7 @@ int hyteg_mesh_create(int dim, int64_t n_verts, const double* coords, int64_t n_
  * 64) for several work splits (float-float and fp32; native fp64 takes the
  * float-float choice), the 2D kernel for tiles of 8, 16, 32 and 64 rows
  * (likewise), timed on two scratch float64 vectors of the level's size
- * (freed before returning); the fastest is kept (choices cached per macro
+ * (freed before returning); the fastest is kept (choices cached per device, macro
  * count and level for the process; see hyteg_autotune_choice).  Meshes built
  * by the solve server only take cached choices: their timings would run
  * among other requests' kernels.

@@ -9,12 +9,12 @@
 // (read before the previous kernel has finished) and one round of loads.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <type_traits>
 #include <vector>
 
 #include "direct.cuh"
 #include "march3d.cuh"
+#include "per_device.h"
 
 namespace hyteg {
 
@@ -173,17 +173,18 @@ template <class P, int MODE, int STRIDE>
 cudaError_t march_attr() {
   using B = March3<P, MODE, STRIDE>;
   static_assert(B::smem_bytes() <= kSmemMax, "the ring does not fit");
-  static std::once_flag once;
-  static cudaError_t err = cudaSuccess;
-  std::call_once(once, [] {
-    err = cudaFuncSetAttribute(k_group<B, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::smem_bytes());
+  static PerDevice set;
+  int value = 0;
+  return set.get(&value, [](int*) {
+    cudaError_t err =
+        cudaFuncSetAttribute(k_group<B, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::smem_bytes());
     if constexpr (STRIDE <= 512) {
       if (err == cudaSuccess)
         err = cudaFuncSetAttribute(k_group<B, kGroupMax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)B::smem_bytes());
     }
+    return err;
   });
-  return err;
 }
 
 template <class P, int MODE, int STRIDE>

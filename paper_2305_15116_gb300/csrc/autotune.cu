@@ -15,8 +15,8 @@ namespace hyteg {
 // range that are read beside the written ones.  On first use of a level size
 // the kernel is timed for each candidate on scratch vectors (the best of two
 // launches each, so that a concurrent workload inflates no candidate in
-// particular) and the fastest list is kept; the choice is cached per (macro
-// count, level, element type) for the process.  Float-float and fp32 are
+// particular) and the fastest list is kept; the choice is cached per (device,
+// macro count, level, element type) for the process.  Float-float and fp32 are
 // timed; native fp64, which the direct kernel takes, reports float-float's
 // choice.  Levels below 2^20 slots take the direct kernel; above n = 64, n/32
 // ranges.
@@ -26,7 +26,7 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
   const int64_t total = L.slots_per_macro * m.n_cells;
   if (total < (int64_t(1) << 20)) return cudaSuccess;
   static std::mutex mu;
-  static std::map<std::array<int64_t, 3>, int> cache;
+  static std::map<std::array<int64_t, 4>, int> cache;
   constexpr int kCand[] = {2, 3, 4, 5, 6, 8};
   void* x = nullptr;
   void* y = nullptr;
@@ -44,7 +44,7 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
     dev_free(m, y);
   };
   for (int dt = 1; dt <= 3 && err == cudaSuccess; ++dt) {
-    const std::array<int64_t, 3> key{m.n_cells, L.n, dt == 3 ? 1 : dt};
+    const std::array<int64_t, 4> key{m.device, m.n_cells, L.n, dt == 3 ? 1 : dt};
     int best = dt == 3 ? L.z_chunks[1] : 0;
     if (best == 0) {
       std::lock_guard<std::mutex> lk(mu);
@@ -117,8 +117,8 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
 // macros: float-float flat from 16 to 64 rows, fp32 best at 16).  On first
 // use of a level size of at least 2^20 slots the apply kernel is timed for
 // 8, 16, 32 and 64 rows (best of two launches after a warm-up) on scratch
-// vectors, float-float and fp32, and the fastest list is kept (cached per macro
-// count, level and element type for the process); native fp64, which the direct
+// vectors, float-float and fp32, and the fastest list is kept (cached per
+// device, macro count, level and element type for the process); native fp64, which the direct
 // kernel takes, reports float-float's choice.  Smaller levels keep the
 // default lists (their kernels take microseconds, and the chunk already
 // shrinks until the level has 16 tiles per SM).
@@ -127,7 +127,7 @@ cudaError_t tiles2d_autotune(Mesh& m, LevelDev& L) {
   const int64_t total = L.slots_per_macro * m.n_cells;
   if (total < (int64_t(1) << 20) || L.n < 64) return cudaSuccess;
   static std::mutex mu;
-  static std::map<std::array<int64_t, 3>, int> cache;
+  static std::map<std::array<int64_t, 4>, int> cache;
   constexpr int kCand[] = {8, 16, 32, 64};
   void* x = nullptr;
   void* y = nullptr;
@@ -145,7 +145,7 @@ cudaError_t tiles2d_autotune(Mesh& m, LevelDev& L) {
     dev_free(m, y);
   };
   for (int dt = 1; dt <= 2 && err == cudaSuccess; ++dt) {
-    const std::array<int64_t, 3> key{m.n_cells, L.n, dt};
+    const std::array<int64_t, 4> key{m.device, m.n_cells, L.n, dt};
     int best = 0;
     {
       std::lock_guard<std::mutex> lk(mu);

@@ -18,10 +18,10 @@
 // (1024 spilled: 156 us; 256: 131, 128: 150), 16 blocks (8: 142 us).  In 3D the
 // launches stay: the gathers are twice as long and need the whole device (a
 // level-5 solve 5.44 against 6.21 ms).
-#include <mutex>
 #include <vector>
 
 #include "direct.cuh"
+#include "per_device.h"
 #include "transfer.cuh"
 
 namespace hyteg {
@@ -207,11 +207,11 @@ __global__ void __launch_bounds__(CTHREADS, 1) k_coarse(const __grid_constant__ 
   }
 }
 
-// Blocks per cluster: 16 where the device places such clusters, else 8.
-int cluster_size() {
-  static std::once_flag once;
-  static int size = 8;
-  std::call_once(once, [] {
+// Blocks per cluster: 16 where the current device places such clusters, else 8.
+cudaError_t cluster_size(int* size) {
+  static PerDevice sizes;
+  return sizes.get(size, [](int* v) {
+    *v = 8;
     if (cudaFuncSetAttribute(k_coarse, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(16);
@@ -222,18 +222,20 @@ int cluster_size() {
       cfg.attrs = at;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k_coarse, &cfg) == cudaSuccess && n > 0) size = 16;
+      if (cudaOccupancyMaxActiveClusters(&n, k_coarse, &cfg) == cudaSuccess && n > 0) *v = 16;
     }
     cudaGetLastError();
+    return cudaSuccess;
   });
-  return size;
 }
 
 }  // namespace
 
 cudaError_t launch_coarse_cycle(Mesh* const* ms, int cnt, int l, const float* const* b, float* const* u,
                                 bool first_done, cudaStream_t s) {
-  const int cluster = cluster_size();
+  int cluster = 8;
+  const cudaError_t ec = cluster_size(&cluster);
+  if (ec != cudaSuccess) return ec;
   for (int i0 = 0; i0 < cnt; i0 += kGroupMax) {
     CoarseArgs g;
     const int k = cnt - i0 < kGroupMax ? cnt - i0 : kGroupMax;
@@ -261,6 +263,9 @@ cudaError_t launch_coarse_cycle(Mesh* const* ms, int cnt, int l, const float* co
   return cudaSuccess;
 }
 
-void coarse_cycle_prepare() { cluster_size(); }
+cudaError_t coarse_cycle_prepare() {
+  int size = 0;
+  return cluster_size(&size);
+}
 
 }  // namespace hyteg

@@ -275,7 +275,7 @@ void march3d_lists(int n, int chunks, int dtype, std::vector<int4>& work, int& s
 cudaError_t set_march(const Mesh& m, LevelDev& L, int dt, int chunks);
 // Time the 3D march on this level for several z-range counts per element
 // type and keep the fastest list (levels of at least 2^20 slots; results are
-// cached per (macro count, level size) for the process).  Synchronous.
+// cached per (device, macro count, level size) for the process).  Synchronous.
 cudaError_t march3d_autotune(Mesh& m, int level);
 // The 2D macro-interior tiles of one macro (same list for every macro):
 // strips of 62 columns from x = 1, rows cut into chunks of `rows`, ordered
@@ -339,7 +339,7 @@ void solver_free(Mesh& m);
 // one launch, l <= Solver::coarse_top (coarse.cu); vectors as vcycle_g.
 cudaError_t launch_coarse_cycle(Mesh* const* ms, int cnt, int l, const float* const* b, float* const* u,
                                 bool first_done, cudaStream_t s);
-void coarse_cycle_prepare();  // before any stream capture
+cudaError_t coarse_cycle_prepare();  // before any stream capture
 // 2D levels of at most so many slots (one V-cycle on 32 macro-triangles at level
 // 10: 781 us without, 757, 734 and 723 us with a limit of 4000, 16000 and 32000
 // slots; with 1024 threads per block 64000 was 10 % slower than 32000)
@@ -392,8 +392,8 @@ cudaError_t launch_sweep3d_group(bool jacobi, const Mesh* const* ms, const int* 
 // the march over an explicit work list (the autotuner's candidates)
 cudaError_t launch_march3d_work(int dtype, const Mesh& m, int level, const March3Work& work, const void* x, void* y,
                                 cudaStream_t s);
-// raises the march kernels' shared-memory limit (once per process; before any
-// stream capture)
+// raises the march kernels' shared-memory limit on the current device (once;
+// before any stream capture)
 cudaError_t apply3d_prepare(int n);
 // ys hold every copy's partial row: the sums over the copies (Dirichlet: x)
 cudaError_t launch_sum_copies3d(const Mesh* const* ms, const int* levels, const double* const* xs, double* const* ys,

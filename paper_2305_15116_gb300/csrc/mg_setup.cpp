@@ -486,7 +486,8 @@ std::string solver_setup(Mesh& m, int max_level, int nu1, int nu2, double omega)
   }
   if (!cl.empty()) {
     if (!(err = upload_vec(m, &sv.coarse, cl)).empty()) return err;
-    coarse_cycle_prepare();
+    const cudaError_t ep = coarse_cycle_prepare();
+    if (ep != cudaSuccess) return std::string("cuda: ") + cudaGetErrorString(ep);
   }
   const cudaError_t e = dev_sync(m);
   if (e != cudaSuccess) return std::string("cuda: set-up: ") + cudaGetErrorString(e);
