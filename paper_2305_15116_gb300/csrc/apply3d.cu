@@ -214,7 +214,8 @@ cudaError_t launch_march_s(const Mesh* const* ms, const int* levels, const void*
     p.md = md ? md[i] : ModeArgs{nullptr, nullptr, 0.0};
     p.n = L.n;
     p.S = L.slots_per_macro;
-    if (w.stride > STRIDE) return cudaErrorInvalidValue;
+    // n >= 4: there are points to march over, and a list that holds them
+    if (w.stride > STRIDE || (w.n_work == 0 && L.n >= 4)) return cudaErrorInvalidValue;
     p.n_march = int64_t(p.n_work) * p.n_pairs;
     const int64_t all = p.n_march + (p.n_march < kOwnIfaceBlocks ? (p.f.n_units + 7) / 8 : 0);
     if (all > 0x7FFFFFFF) return cudaErrorInvalidValue;

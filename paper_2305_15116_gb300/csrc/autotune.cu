@@ -75,13 +75,14 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
       }
       float best_ms = 0.0f;
       for (int c : kCand) {
-        if ((err = set_march(m, L, dt, c)) != cudaSuccess) break;
-        if ((err = dev_sync(m)) != cudaSuccess) break;
+        March3Work work;
+        if ((err = make_march(m, L.n, dt, c, work)) != cudaSuccess) break;
+        err = dev_sync(m);
         float ms = 0.0f;
         const int first = c == kCand[0] ? 0 : 1;  // one warm-up launch per element type
         for (int rep = first; rep < 3 && err == cudaSuccess; ++rep) {
           if ((err = cudaEventRecord(e0, s)) != cudaSuccess) break;
-          if ((err = launch_march3d_work(dt, m, level, L.march[dt], x, y, s)) != cudaSuccess) break;
+          if ((err = launch_march3d_work(dt, m, level, work, x, y, s)) != cudaSuccess) break;
           if ((err = cudaEventRecord(e1, s)) != cudaSuccess) break;
           if ((err = cudaEventSynchronize(e1)) != cudaSuccess) break;
           float t = 0.0f;
@@ -89,6 +90,7 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
           if (rep == 1 || (rep > 1 && t < ms)) ms = t;
         }
         const cudaError_t ef = cudaStreamSynchronize(s);
+        dev_free(m, work.work);
         if (err == cudaSuccess) err = ef;
         if (err != cudaSuccess) break;
         if (best == 0 || ms < best_ms) {
@@ -102,6 +104,10 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
     }
     if ((err = set_march(m, L, dt, best)) != cudaSuccess) break;
     L.z_chunks[dt] = best;
+  }
+  if (err == cudaErrorMemoryAllocation) {  // no room for a list: the level keeps the one it has
+    cudaGetLastError();
+    err = cudaSuccess;
   }
   if (err == cudaSuccess) err = dev_sync(m);
   cleanup();

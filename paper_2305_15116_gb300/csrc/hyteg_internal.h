@@ -268,10 +268,13 @@ void set_last_error(const std::string& msg);
 std::string build_topology(Mesh& m);
 std::string build_level(Mesh& m, int level, LevelDev& out);
 // z-ranges (-, z0, z1, -): a macro cut into `chunks` ranges of about equal
-// point counts
+// slice counts
 std::vector<int4> z_ranges(int n, int chunks);
-// the work list of the 3D march for `chunks` z-ranges, built and uploaded
+// the work list of the 3D march for `chunks` z-ranges; on the device (`out` only
+// if that succeeds), and as the level's list in place of the one it had (which
+// stays if that fails)
 void march3d_lists(int n, int chunks, int dtype, std::vector<int4>& work, int& stride);
+cudaError_t make_march(const Mesh& m, int n, int dt, int chunks, March3Work& out);
 cudaError_t set_march(const Mesh& m, LevelDev& L, int dt, int chunks);
 // Time the 3D march on this level for several z-range counts per element
 // type and keep the fastest list (levels of at least 2^20 slots; results are

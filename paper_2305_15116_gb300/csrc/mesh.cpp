@@ -299,21 +299,31 @@ std::vector<int4> z_ranges(int n, int chunks) {
   return r;
 }
 
-cudaError_t set_march(const Mesh& m, LevelDev& L, int dt, int chunks) {
+cudaError_t make_march(const Mesh& m, int n, int dt, int chunks, March3Work& out) {
   std::vector<int4> w;
-  March3Work& k = L.march[dt];
-  march3d_lists(L.n, chunks, dt, w, k.stride);
-  dev_free(m, k.work);
-  k.work = nullptr;
+  March3Work k;
+  march3d_lists(n, chunks, dt, w, k.stride);
   k.n_work = int(w.size());
-  if (w.empty()) return cudaSuccess;
-  const cudaError_t e = dev_alloc(m, (void**)&k.work, w.size() * sizeof(int4));
-  if (e != cudaSuccess) {
-    k.work = nullptr;
-    k.n_work = 0;
-    return e;
+  if (!w.empty()) {
+    cudaError_t e = dev_alloc(m, (void**)&k.work, w.size() * sizeof(int4));
+    if (e != cudaSuccess) return e;
+    e = dev_upload(m, k.work, w.data(), w.size() * sizeof(int4));
+    if (e != cudaSuccess) {
+      dev_free(m, k.work);
+      return e;
+    }
   }
-  return dev_upload(m, k.work, w.data(), w.size() * sizeof(int4));
+  out = k;
+  return cudaSuccess;
+}
+
+cudaError_t set_march(const Mesh& m, LevelDev& L, int dt, int chunks) {
+  March3Work k;
+  const cudaError_t e = make_march(m, L.n, dt, chunks, k);
+  if (e != cudaSuccess) return e;
+  dev_free(m, L.march[dt].work);
+  L.march[dt] = k;
+  return cudaSuccess;
 }
 
 void free_level(const Mesh& m, LevelDev& L) {

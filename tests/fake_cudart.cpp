@@ -59,6 +59,7 @@ void fake_fail_malloc(long after, size_t bytes) {
   malloc_left = after;
   fail_bytes = bytes;
 }
+int fake_malloc_armed() { return malloc_left >= 0; }
 void fake_fail_new(long after) { new_left = after; }
 void fake_clear_log() { log_.clear(); }
 const char* fake_log() { return log_.c_str(); }  // kernel, device, grid, block, dynamic shared memory, cluster
