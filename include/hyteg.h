@@ -73,8 +73,8 @@ extern "C" {
                                 float-float range (zero or 2^-80 <= |x| < 2^64)
                                 are recomputed with native fp64 FMAs in the same
                                 launch, and levels with a stencil whose largest
-                                weight leaves 2^-20 .. 2^14 run the native
-                                kernels */
+                                weight leaves 2^-20 .. 2^14, and 3D levels
+                                above 9, run the native kernels */
 #define HYTEG_F32       2    /* float32 vectors, fp32 FMA arithmetic */
 #define HYTEG_F64_IEEE  3    /* float64 vectors, native fp64 FMA arithmetic */
 
@@ -156,8 +156,9 @@ int hyteg_dof_map(const hyteg_mesh* mesh, int level, int64_t* global_id);
  *   y       device, [n_slots]; every slot is written; must not overlap x
  *   stream  cudaStream_t as void*
  * Asynchronous.  No allocation.  Deterministic: the same inputs give bitwise
- * the same outputs.  Errors: HYTEG_EINVAL (null, x == y, dtype),
- * HYTEG_ESTATE (level not refined), HYTEG_ECUDA (launch failure). */
+ * the same outputs.  Errors: HYTEG_EINVAL (null, x == y, dtype, a 3D level
+ * above 11, whose macros hold more than 2^32 slots), HYTEG_ESTATE (level not
+ * refined), HYTEG_ECUDA (launch failure). */
 int hyteg_apply(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y,
                 void* stream);
 

@@ -52,6 +52,19 @@ int hyteg::check_level(const hyteg_mesh* mesh, int level) {
 
 extern "C" {
 
+namespace {
+
+// check_level, and the levels whose products the kernels take: in 3D a macro's
+// slots are counted in 32 bits (level 12: 1.1e10).
+int check_product(const hyteg_mesh* mesh, int level) {
+  if (int r = check_level(mesh, level)) return r;
+  if (mesh->m.dim == 3 && level > hyteg::kMaxProductLevel3)
+    return fail(HYTEG_EINVAL, "3D products take levels up to " + std::to_string(hyteg::kMaxProductLevel3));
+  return HYTEG_OK;
+}
+
+}  // namespace
+
 int hyteg_mesh_create(int dim, int64_t n_verts, const double* coords, int64_t n_cells, const int64_t* cells,
                       int bc, hyteg_mesh** out) {
   if (!out) return fail(HYTEG_EINVAL, "out is NULL");
@@ -180,7 +193,7 @@ int hyteg_dof_map(const hyteg_mesh* mesh, int level, int64_t* global_id) {
 
 int hyteg_apply_timed(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream,
                       void* ev_begin, void* ev_mid, void* ev_end) {
-  if (int r = check_level(mesh, level)) return r;
+  if (int r = check_product(mesh, level)) return r;
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   if (!x || !y) return fail(HYTEG_EINVAL, "x or y is NULL");
   const hyteg::Mesh& m = mesh->m;
@@ -205,7 +218,7 @@ int hyteg_apply(const hyteg_mesh* mesh, int level, int dtype, const void* x, voi
 }
 
 int hyteg_apply_partial(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream) {
-  if (int r = check_level(mesh, level)) return r;
+  if (int r = check_product(mesh, level)) return r;
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   if (!x || !y) return fail(HYTEG_EINVAL, "x or y is NULL");
   const hyteg::Mesh& m = mesh->m;
@@ -226,7 +239,7 @@ int hyteg_apply_batch(const hyteg_mesh* const* meshes, const int* levels, int dt
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   // validate everything before the first launch
   for (int i = 0; i < count; ++i) {
-    if (int r = check_level(meshes[i], levels[i])) return r;
+    if (int r = check_product(meshes[i], levels[i])) return r;
     if (!xs[i] || !ys[i]) return fail(HYTEG_EINVAL, "x or y is NULL (entry " + std::to_string(i) + ")");
     const hyteg::Mesh& m = meshes[i]->m;
     const size_t bytes = size_t(m.n_cells) * size_t(hyteg::slots_per_macro(m.dim, levels[i])) * elem_size(dtype);
@@ -264,7 +277,7 @@ int hyteg_apply_batch(const hyteg_mesh* const* meshes, const int* levels, int dt
 }
 
 int hyteg_apply_host(hyteg_mesh* mesh, int level, int dtype, const void* x_host, void* y_host, void* stream) {
-  if (int r = check_level(mesh, level)) return r;
+  if (int r = check_product(mesh, level)) return r;
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   if (!x_host || !y_host) return fail(HYTEG_EINVAL, "x_host or y_host is NULL");
   hyteg::Mesh& m = mesh->m;
@@ -298,7 +311,7 @@ int hyteg_apply_host(hyteg_mesh* mesh, int level, int dtype, const void* x_host,
 
 int hyteg_apply_host_batch(hyteg_mesh* mesh, int level, int dtype, const void* const* x_hosts,
                            void* const* y_hosts, int count, void* stream) {
-  if (int r = check_level(mesh, level)) return r;
+  if (int r = check_product(mesh, level)) return r;
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   if (count < 0 || (count > 0 && (!x_hosts || !y_hosts))) return fail(HYTEG_EINVAL, "bad batch");
   for (int i = 0; i < count; ++i)

@@ -379,6 +379,8 @@ cudaError_t launch_sweep2d_group(bool jacobi, const Mesh* const* ms, const int* 
                                  void* const* out, int count, cudaStream_t s);
 // 2D levels of at most so many slots take the direct kernel (interior2d.cu)
 constexpr int64_t kDirect2MaxSlots = 3 * (int64_t(1) << 17);
+// the finest level of 3D products (32-bit slots inside a macro)
+constexpr int kMaxProductLevel3 = 11;
 // Levels whose vectors the direct 3D kernel takes (LevelDev::direct3), and the
 // levels with its point table (which native fp64 always uses).
 constexpr int kDirect3MaxN = 64;
