@@ -9,30 +9,31 @@
 
 #include "arith.cuh"
 #include "hyteg_internal.h"
+#include "modes.cuh"
 
 namespace hyteg {
 
 // 2D macro-interior row of the point at p (row length len = n + 1 - y):
 // weights w[0..6] in the order S, SE, W, C, E, NW, N.  Row y+1 starts len
 // slots after row y, row y-1 len + 1 slots before it.
-__device__ __forceinline__ double native_row2d(const double* __restrict__ p, int len,
+__device__ __forceinline__ double native_row2d(const double* p, int len,
                                                    const double* __restrict__ w) {
-  double a = __dmul_rn(__ldg(w + 3), __ldg(p));
-  a = __fma_rn(__ldg(w + 4), __ldg(p + 1), a);
-  a = __fma_rn(__ldg(w + 2), __ldg(p - 1), a);
-  a = __fma_rn(__ldg(w + 6), __ldg(p + len), a);
-  a = __fma_rn(__ldg(w + 5), __ldg(p + len - 1), a);
-  a = __fma_rn(__ldg(w + 0), __ldg(p - len - 1), a);
-  a = __fma_rn(__ldg(w + 1), __ldg(p - len), a);
+  double a = __dmul_rn(__ldg(w + 3), ld<false>(p));
+  a = __fma_rn(__ldg(w + 4), ld<false>(p + 1), a);
+  a = __fma_rn(__ldg(w + 2), ld<false>(p - 1), a);
+  a = __fma_rn(__ldg(w + 6), ld<false>(p + len), a);
+  a = __fma_rn(__ldg(w + 5), ld<false>(p + len - 1), a);
+  a = __fma_rn(__ldg(w + 0), ld<false>(p - len - 1), a);
+  a = __fma_rn(__ldg(w + 1), ld<false>(p - len), a);
   return a;
 }
 
 // Whether that row reads an input outside the float-float range (a walker
 // learns it for its whole tile only).
-__device__ __forceinline__ bool row2d_out_of_range(const double* __restrict__ p, int len) {
-  return !(ff_in_range(__ldg(p)) && ff_in_range(__ldg(p + 1)) && ff_in_range(__ldg(p - 1)) &&
-           ff_in_range(__ldg(p + len)) && ff_in_range(__ldg(p + len - 1)) && ff_in_range(__ldg(p - len - 1)) &&
-           ff_in_range(__ldg(p - len)));
+__device__ __forceinline__ bool row2d_out_of_range(const double* p, int len) {
+  return !(ff_in_range(ld<false>(p)) && ff_in_range(ld<false>(p + 1)) && ff_in_range(ld<false>(p - 1)) &&
+           ff_in_range(ld<false>(p + len)) && ff_in_range(ld<false>(p + len - 1)) && ff_in_range(ld<false>(p - len - 1)) &&
+           ff_in_range(ld<false>(p - len)));
 }
 
 // Slot of lattice point (x, y, z) inside a 3D macro array of level n = 2^L.
@@ -45,7 +46,7 @@ __device__ __forceinline__ int64_t fb_slot3(int n, int x, int y, int z) {
 // (centre, the six in-slice neighbours, four of slice z+1, four of slice z-1,
 // in the order of the kernels' weight slots).  Neighbours outside the macro
 // carry weight 0 in every class stencil and are skipped.
-__device__ __forceinline__ double native_row3d(const double* __restrict__ xm, int n, int px, int py, int pz,
+__device__ __forceinline__ double native_row3d(const double* xm, int n, int px, int py, int pz,
                                                    const double* __restrict__ w) {
   const signed char off[NW3][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0},
                                    {1, -1, 0}, {-1, 1, 0}, {0, 0, 1},  {-1, 0, 1}, {0, -1, 1},
@@ -55,7 +56,7 @@ __device__ __forceinline__ double native_row3d(const double* __restrict__ xm, in
     const int qx = px + off[k][0], qy = py + off[k][1], qz = pz + off[k][2];
     if (qx < 0 || qy < 0 || qz < 0 || qx + qy + qz > n) continue;
     const double wk = __ldg(w + k);
-    if (wk != 0.0) a = __fma_rn(wk, __ldg(xm + fb_slot3(n, qx, qy, qz)), a);
+    if (wk != 0.0) a = __fma_rn(wk, ld<false>(xm + fb_slot3(n, qx, qy, qz)), a);
   }
   return a;
 }

@@ -13,6 +13,7 @@
 
 #include "group.cuh"
 #include "hyteg_internal.h"
+#include "modes.cuh"
 
 namespace hyteg {
 
@@ -67,7 +68,7 @@ struct SumItems2 {
     if (it.z + (int)threadIdx.x >= it.w) return;
     double acc = 0.0;
     if (pr.boundary) {
-      acc = __ldg(p.x + slot_of(0));
+      acc = ld<false>(p.x + slot_of(0));
     } else {
       for (int i = 0; i < pr.inc_count; ++i) acc += p.y[slot_of(i)];
     }

@@ -106,8 +106,8 @@ struct Thr2 {
 // The work of one block of an apply / sweep launch over one mesh (block =
 // the block's index within that mesh's part of the launch).
 template <class P, int MODE>
-__device__ __forceinline__ void apply2d_block(int block, const typename P::T* __restrict__ x,
-                                              typename P::T* __restrict__ y, const int4* __restrict__ tiles,
+__device__ __forceinline__ void apply2d_block(int block, const typename P::T* x,
+                                              typename P::T* y, const int4* __restrict__ tiles,
                                               int n_tiles, int64_t n_warps, int64_t S, int n, const StencilPtr& st,
                                               const IfItem* __restrict__ items, int n_items,
                                               const Inc* __restrict__ incs,
@@ -136,9 +136,9 @@ __device__ __forceinline__ void apply2d_block(int block, const typename P::T* __
   const int4 t = tiles[warp - m * n_tiles];
   const int ca = t.x - 1 + 2 * lane;  // column A; column B = ca + 1
   const int cb = ca + 1;
-  const T* __restrict__ xm = x + m * S;
-  T* __restrict__ ym = y + m * S;
-  const T* __restrict__ bm = SWEEP ? static_cast<const T*>(md.b) + m * S : nullptr;
+  const T* xm = x + m * S;
+  T* ym = y + m * S;
+  const T* bm = SWEEP ? static_cast<const T*>(md.b) + m * S : nullptr;
   // inverse diagonal of the macro's interior points, rounded as the set-up's
   const T dint = MODE == MODE_JACOBI ? (T)(1.0 / __ldg(st.d + m * (int64_t)(NCLS2 * NW2) + C2)) : T(0);
 
@@ -159,8 +159,8 @@ __device__ __forceinline__ void apply2d_block(int block, const typename P::T* __
   const bool wa = lane >= 1, wbb = lane <= 30;   // lane 0's A and lane 31's B are halo
   int off_s = (t.y - 1) * (n + 2) - ((t.y - 1) * t.y) / 2;  // the row being staged
   int len_s = n + 2 - t.y;
-  const T* __restrict__ xa = xm + ca;
-  const T* __restrict__ ba = SWEEP ? bm + ca : nullptr;
+  const T* xa = xm + ca;
+  const T* ba = SWEEP ? bm + ca : nullptr;
   // fp32: on the rows where a lane's two columns form an aligned pair (the
   // same for every lane of the warp) one 8-byte copy per vector and one
   // store take both (the load/store queue bounds these kernels; in the
@@ -234,7 +234,7 @@ __device__ __forceinline__ void apply2d_block(int block, const typename P::T* __
   auto take = [&](int k, auto slot_c) -> Row<P> { return take_g(k, slot_c, Guarded{}); };
   int off_o = t.y * (n + 2) - (t.y * (t.y + 1)) / 2;  // the row being written
   int len_o = n + 1 - t.y;
-  T* __restrict__ ya = ym + ca;
+  T* ya = ym + ca;
   typename P::Mark mk = P::mark0();
   // output row r_{k-1} from (below, centre, above) = rows r_{k-2}, r_{k-1}, r_k
   auto step = [&](const Row<P>& lo, const Row<P>& ce, const Row<P>& hi, int k) {
@@ -309,10 +309,14 @@ __device__ __forceinline__ void apply2d_block(int block, const typename P::T* __
     // its two columns of the tile again, in native fp64 from memory
     if (P::marked(mk)) {
       const double* wd = st.d + wb;
+      // through an opaque copy of the pointer: addresses shared with the walk
+      // would cost it registers (level 11, 32 macros: 260 against 255 us)
+      const T* xf = xm;
+      asm volatile("" : "+l"(xf));
       Cursor rw;
       rw.init(n, t.y);
       for (int r = t.y; r < t.z; ++r) {
-        const double* const xr = xm + rw.off;
+        const double* const xr = xf + rw.off;
         if (wa && ca < rw.len - 1 && row2d_out_of_range(xr + ca, rw.len))
           ym[rw.off + ca] = native_row2d(xr + ca, rw.len, wd);
         if (wbb && cb < rw.len - 1 && row2d_out_of_range(xr + cb, rw.len))
@@ -331,8 +335,7 @@ struct MinBlocks2 {
 };
 
 template <class P, int MODE>
-__global__ void __launch_bounds__(Thr2<MODE>::value, MinBlocks2<P>::value) k_interior2d(const typename P::T* __restrict__ x,
-                                                          typename P::T* __restrict__ y,
+__global__ void __launch_bounds__(Thr2<MODE>::value, MinBlocks2<P>::value) k_interior2d(const typename P::T* x, typename P::T* y,
                                                           const int4* __restrict__ tiles, int n_tiles,
                                                           int64_t n_warps, int64_t S, int n, StencilPtr st,
                                                           const IfItem* __restrict__ items, int n_items,

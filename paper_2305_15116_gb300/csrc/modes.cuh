@@ -26,7 +26,9 @@ struct ModeArgs {
 // written by other blocks of the same launch are seen after a barrier between
 // them.  Not the read-only path: a kernel may start before the one that writes
 // the vector has finished (group.cuh), and the code generator may move a
-// read-only load, which it takes for invariant, above the wait.
+// read-only load, which it takes for invariant, above the wait.  For the same
+// reason no vector of such a kernel is a __restrict__ pointer: that promises
+// that nothing else, the wait included, changes what it points to.
 template <bool CG, class T>
 __device__ __forceinline__ T ld(const T* p) {
   if constexpr (CG)

@@ -203,8 +203,8 @@ struct PartialDiff {
       unpack<DIM>(p.lpts[i - cell * S], q);
       const int cls = pclass<DIM>(n, q);
       const double* __restrict__ w = p.st + (cell * NCLS + cls) * NW;
-      const double* __restrict__ um = p.u + cell * S;
-      const double* __restrict__ lm = p.ulo ? p.ulo + cell * S : nullptr;
+      const double* um = p.u + cell * S;
+      const double* lm = p.ulo ? p.ulo + cell * S : nullptr;
       const double uc = um[i - cell * S];
       const double lc = lm ? lm[i - cell * S] : 0.0;
       double acc = 0.0;

@@ -20,6 +20,7 @@
 #include "fallback.cuh"
 #include "group.cuh"
 #include "hyteg_internal.h"
+#include "modes.cuh"
 
 namespace hyteg {
 
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(P2THREADS) k_p2_rows(const typename P::T* __re
 // Edge DoFs on coarse edges: sum the copies' partial rows in ascending macro
 // order and write the sum to every copy (Dirichlet edges: y = x).
 template <class T>
-__device__ __forceinline__ void p2_edge_reduce(const T* __restrict__ x, T* __restrict__ y, const int4& it,
+__device__ __forceinline__ void p2_edge_reduce(const T* x, T* y, const int4& it,
                                                 const Prim* __restrict__ prims, const Inc* __restrict__ incs,
                                                 const Geo& G) {
   const int t = it.y + threadIdx.x;
@@ -453,7 +454,7 @@ __device__ __forceinline__ void p2_edge_reduce(const T* __restrict__ x, T* __res
   };
   T acc = T(0);
   if (p.boundary) {
-    acc = __ldg(x + slot_of(0));
+    acc = ld<false>(x + slot_of(0));
   } else {
     for (int i = 0; i < p.inc_count; ++i) acc += y[slot_of(i)];
   }
@@ -463,7 +464,7 @@ __device__ __forceinline__ void p2_edge_reduce(const T* __restrict__ x, T* __res
 // Vertex DoFs on coarse vertices and edges: as the P1 reduction, in the P2
 // macro blocks.
 template <class T>
-__device__ __forceinline__ void p2_vertex_reduce(const T* __restrict__ x, T* __restrict__ y, const int4& it,
+__device__ __forceinline__ void p2_vertex_reduce(const T* x, T* y, const int4& it,
                                                 const Prim* __restrict__ prims, const Inc* __restrict__ incs,
                                                 const Geo& G) {
   const int a = it.z + threadIdx.x;
@@ -487,16 +488,17 @@ __device__ __forceinline__ void p2_vertex_reduce(const T* __restrict__ x, T* __r
   };
   T acc = T(0);
   if (p.boundary) {
-    acc = __ldg(x + slot_of(0));
+    acc = ld<false>(x + slot_of(0));
   } else {
     for (int i = 0; i < p.inc_count; ++i) acc += y[slot_of(i)];
   }
   for (int i = 0; i < p.inc_count; ++i) y[slot_of(i)] = acc;
 }
 
-// Both reductions in one launch, which is placed while the row kernel drains.
+// Both reductions in one launch, which is placed while the row kernel drains:
+// y is read after pdl_wait only (plain pointers, modes.cuh).
 template <class T>
-__global__ void __launch_bounds__(128) k_p2_reduce(const T* __restrict__ x, T* __restrict__ y,
+__global__ void __launch_bounds__(128) k_p2_reduce(const T* x, T* y,
                                                    const int4* __restrict__ v_items, int n_v,
                                                    const int4* __restrict__ e_items, const Prim* __restrict__ prims,
                                                    const Inc* __restrict__ incs, Geo G) {
