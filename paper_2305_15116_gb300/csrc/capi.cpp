@@ -50,6 +50,10 @@ int hyteg::check_level(const hyteg_mesh* mesh, int level) {
   return HYTEG_OK;
 }
 
+// ends an entry whose host code may run out of memory: nothing is thrown at a C caller
+#define HYTEG_CATCH \
+  catch (const std::bad_alloc&) { return fail(HYTEG_ENOMEM, "host allocation failed"); }
+
 extern "C" {
 
 namespace {
@@ -192,7 +196,7 @@ int hyteg_dof_map(const hyteg_mesh* mesh, int level, int64_t* global_id) {
 }
 
 int hyteg_apply_timed(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream,
-                      void* ev_begin, void* ev_mid, void* ev_end) {
+                      void* ev_begin, void* ev_mid, void* ev_end) try {
   if (int r = check_product(mesh, level)) return r;
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   if (!x || !y) return fail(HYTEG_EINVAL, "x or y is NULL");
@@ -211,13 +215,13 @@ int hyteg_apply_timed(const hyteg_mesh* mesh, int level, int dtype, const void* 
   if (ev_end && (e = cudaEventRecord(static_cast<cudaEvent_t>(ev_end), s)) != cudaSuccess)
     return cuda_fail(e, "cudaEventRecord");
   return HYTEG_OK;
-}
+} HYTEG_CATCH
 
 int hyteg_apply(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream) {
   return hyteg_apply_timed(mesh, level, dtype, x, y, stream, nullptr, nullptr, nullptr);
 }
 
-int hyteg_apply_partial(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream) {
+int hyteg_apply_partial(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream) try {
   if (int r = check_product(mesh, level)) return r;
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   if (!x || !y) return fail(HYTEG_EINVAL, "x or y is NULL");
@@ -229,10 +233,10 @@ int hyteg_apply_partial(const hyteg_mesh* mesh, int level, int dtype, const void
   const char* what = "";
   const cudaError_t e = hyteg::launch_apply_partial(m, level, dtype, x, y, static_cast<cudaStream_t>(stream), &what);
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, what);
-}
+} HYTEG_CATCH
 
 int hyteg_apply_batch(const hyteg_mesh* const* meshes, const int* levels, int dtype, const void* const* xs,
-                      void* const* ys, int count, void* stream) {
+                      void* const* ys, int count, void* stream) try {
   if (count < 0) return fail(HYTEG_EINVAL, "count < 0");
   if (count == 0) return HYTEG_OK;
   if (!meshes || !levels || !xs || !ys) return fail(HYTEG_EINVAL, "NULL array");
@@ -274,7 +278,7 @@ int hyteg_apply_batch(const hyteg_mesh* const* meshes, const int* levels, int dt
     if (e != cudaSuccess) return cuda_fail(e, "batched 2D apply kernel");
   }
   return HYTEG_OK;
-}
+} HYTEG_CATCH
 
 int hyteg_apply_host(hyteg_mesh* mesh, int level, int dtype, const void* x_host, void* y_host, void* stream) {
   if (int r = check_product(mesh, level)) return r;
@@ -310,7 +314,7 @@ int hyteg_apply_host(hyteg_mesh* mesh, int level, int dtype, const void* x_host,
 }
 
 int hyteg_apply_host_batch(hyteg_mesh* mesh, int level, int dtype, const void* const* x_hosts,
-                           void* const* y_hosts, int count, void* stream) {
+                           void* const* y_hosts, int count, void* stream) try {
   if (int r = check_product(mesh, level)) return r;
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
   if (count < 0 || (count > 0 && (!x_hosts || !y_hosts))) return fail(HYTEG_EINVAL, "bad batch");
@@ -397,7 +401,7 @@ int hyteg_apply_host_batch(hyteg_mesh* mesh, int level, int dtype, const void* c
   cleanup();
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
   return HYTEG_OK;
-}
+} HYTEG_CATCH
 
 int hyteg_slot_coords(const hyteg_mesh* mesh, int level, double* xyz) {
   if (int r = check_host_level(mesh, level)) return r;
@@ -455,35 +459,35 @@ int check_solver(const hyteg_mesh* mesh, int level, int min_level) {
 }  // namespace
 
 int hyteg_restrict(const hyteg_mesh* mesh, int fine_level, int dtype, const void* r_fine, void* b_coarse,
-                   void* stream) {
+                   void* stream) try {
   if (int r = check_solver(mesh, fine_level, 1)) return r;
   if (dtype != HYTEG_F64 && dtype != HYTEG_F32) return fail(HYTEG_EINVAL, "dtype must be HYTEG_F64 or HYTEG_F32");
   if (!r_fine || !b_coarse) return fail(HYTEG_EINVAL, "NULL vector");
   const cudaError_t e =
       hyteg::mg_restrict(mesh->m, fine_level, dtype, r_fine, b_coarse, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, "restriction");
-}
+} HYTEG_CATCH
 
 int hyteg_prolong_add(const hyteg_mesh* mesh, int fine_level, int dtype, const void* e_coarse, void* u_fine,
-                      void* stream) {
+                      void* stream) try {
   if (int r = check_solver(mesh, fine_level, 1)) return r;
   if (dtype != HYTEG_F64 && dtype != HYTEG_F32) return fail(HYTEG_EINVAL, "dtype must be HYTEG_F64 or HYTEG_F32");
   if (!e_coarse || !u_fine) return fail(HYTEG_EINVAL, "NULL vector");
   const cudaError_t e =
       hyteg::mg_prolong_add(mesh->m, fine_level, dtype, e_coarse, u_fine, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, "prolongation");
-}
+} HYTEG_CATCH
 
-int hyteg_vcycle(hyteg_mesh* mesh, int level, int dtype, const void* b, void* u, void* stream) {
+int hyteg_vcycle(hyteg_mesh* mesh, int level, int dtype, const void* b, void* u, void* stream) try {
   if (int r = check_solver(mesh, level, 0)) return r;
   if (dtype != HYTEG_F64 && dtype != HYTEG_F32) return fail(HYTEG_EINVAL, "dtype must be HYTEG_F64 or HYTEG_F32");
   if (!b || !u) return fail(HYTEG_EINVAL, "NULL vector");
   const cudaError_t e = hyteg::mg_vcycle(mesh->m, level, dtype, b, u, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, "V-cycle");
-}
+} HYTEG_CATCH
 
 int hyteg_solve(hyteg_mesh* mesh, int level, int mode, const double* b, double* u, double rtol, int max_iter,
-                void* stream, int* iters, double* relres) {
+                void* stream, int* iters, double* relres) try {
   if (int r = check_solver(mesh, level, 0)) return r;
   if (mode != HYTEG_SOLVE_F64 && mode != HYTEG_SOLVE_MIXED) return fail(HYTEG_EINVAL, "unknown mode");
   if (!b || !u || !iters || !relres) return fail(HYTEG_EINVAL, "NULL argument");
@@ -491,10 +495,10 @@ int hyteg_solve(hyteg_mesh* mesh, int level, int mode, const double* b, double* 
   const cudaError_t e = hyteg::mg_solve(mesh->m, level, mode, b, u, nullptr, rtol, max_iter,
                                         static_cast<cudaStream_t>(stream), iters, relres);
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, "solve");
-}
+} HYTEG_CATCH
 
 int hyteg_solve_two_part(hyteg_mesh* mesh, int level, int mode, const double* b, double* u, double* u_lo,
-                         double rtol, int max_iter, void* stream, int* iters, double* relres) {
+                         double rtol, int max_iter, void* stream, int* iters, double* relres) try {
   if (int r = check_solver(mesh, level, 0)) return r;
   if (mode != HYTEG_SOLVE_F64 && mode != HYTEG_SOLVE_MIXED) return fail(HYTEG_EINVAL, "unknown mode");
   if (!b || !u || !u_lo || !iters || !relres) return fail(HYTEG_EINVAL, "NULL argument");
@@ -503,11 +507,11 @@ int hyteg_solve_two_part(hyteg_mesh* mesh, int level, int mode, const double* b,
   const cudaError_t e = hyteg::mg_solve(mesh->m, level, mode, b, u, u_lo, rtol, max_iter,
                                         static_cast<cudaStream_t>(stream), iters, relres);
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, "solve");
-}
+} HYTEG_CATCH
 
 int hyteg_solve_two_part_group(hyteg_mesh* const* meshes, int count, int level, int mode, const double* const* b,
                                double* const* u, double* const* u_lo, double rtol, int max_iter, void* stream,
-                               int* iters, double* relres) {
+                               int* iters, double* relres) try {
   if (count < 1) return fail(HYTEG_EINVAL, "count < 1");
   if (!meshes || !b || !u || !u_lo || !iters || !relres) return fail(HYTEG_EINVAL, "NULL argument");
   if (mode != HYTEG_SOLVE_F64 && mode != HYTEG_SOLVE_MIXED) return fail(HYTEG_EINVAL, "unknown mode");
@@ -529,7 +533,7 @@ int hyteg_solve_two_part_group(hyteg_mesh* const* meshes, int count, int level, 
   const cudaError_t e = hyteg::mg_solve_group(ms.data(), count, level, mode, b, u, u_lo, rtol, max_iter, s, iters,
                                               relres);
   return e == cudaSuccess ? HYTEG_OK : cuda_fail(e, "group solve");
-}
+} HYTEG_CATCH
 
 int hyteg_p2_num_slots(const hyteg_mesh* mesh, int level, int64_t* n_slots, int64_t* n_global) {
   if (int r = check_host_level(mesh, level)) return r;
@@ -552,7 +556,7 @@ int hyteg_p2_dof_map(const hyteg_mesh* mesh, int level, int64_t* global_id) {
 }
 
 int hyteg_p2_apply_timed(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream,
-                         void* ev_begin, void* ev_mid, void* ev_end) {
+                         void* ev_begin, void* ev_mid, void* ev_end) try {
   if (int r = check_level(mesh, level)) return r;
   if (mesh->m.dim != 2) return fail(HYTEG_EINVAL, "the P2 operator is built for 2D meshes");
   if (!valid_dtype(dtype)) return fail(HYTEG_EINVAL, "unknown dtype");
@@ -572,7 +576,7 @@ int hyteg_p2_apply_timed(const hyteg_mesh* mesh, int level, int dtype, const voi
   if (ev_end && (e = cudaEventRecord(static_cast<cudaEvent_t>(ev_end), s)) != cudaSuccess)
     return cuda_fail(e, "cudaEventRecord");
   return HYTEG_OK;
-}
+} HYTEG_CATCH
 
 int hyteg_p2_apply(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y, void* stream) {
   return hyteg_p2_apply_timed(mesh, level, dtype, x, y, stream, nullptr, nullptr, nullptr);

@@ -16,6 +16,7 @@
 // copies of every coarse interface point and zeroes the Dirichlet rows.
 #include <algorithm>
 #include <cmath>
+#include <new>
 #include <vector>
 
 #include "transfer.cuh"
@@ -909,7 +910,12 @@ cudaError_t vcycle_own(Mesh* const* ms, int cnt, int l, cudaStream_t s, bool fir
   if (!ge[l]) {
     cudaGraph_t graph = nullptr;
     HY_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    const cudaError_t e = vcycle_g<T>(ms, 1, l, b.data(), u.data(), s, first_done);
+    cudaError_t e;
+    try {
+      e = vcycle_g<T>(ms, 1, l, b.data(), u.data(), s, first_done);
+    } catch (const std::bad_alloc&) {  // the capture ends all the same
+      e = cudaErrorMemoryAllocation;
+    }
     const cudaError_t e2 = cudaStreamEndCapture(s, &graph);
     if (e != cudaSuccess || e2 != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);
