@@ -110,9 +110,9 @@ int hyteg_mesh_create(int dim, int64_t n_verts, const double* coords, int64_t n_
  * tables with cudaMalloc (size O(cells * levels + interface primitives)),
  * owned by the mesh.  Synchronous.  May be called again with a larger level.
  * Levels of at least 2^20 slots are autotuned here: the 3D kernel (8 < n <=
- * 64) for several work splits (float-float and fp32; native fp64 takes the
- * float-float choice), the 2D kernel for tiles of 8, 16, 32 and 64 rows
- * (likewise), timed on two scratch float64 vectors of the level's size
+ * 64) for several work splits, the 2D kernel for tiles of 8, 16, 32 and 64
+ * rows (float-float and fp32: the native fp64 kernels of these levels have
+ * neither), timed on two scratch float64 vectors of the level's size
  * (freed before returning); the fastest is kept (choices cached per device, macro
  * count and level for the process; see hyteg_autotune_choice).  Meshes built
  * by the solve server only take cached choices: their timings would run
@@ -127,6 +127,7 @@ int hyteg_mesh_refine(hyteg_mesh* mesh, int max_level);
  * 2^20 slots).  2D: the rows per macro-interior tile (8, 16, 32 or 64), timed
  * on levels of at least 2^20 slots; 0 when the level keeps the default
  * tiles (64 rows for float64, 16 for fp32, fewer on levels with few tiles).
+ * HYTEG_F64_IEEE reports the choice of HYTEG_F64.
  * Errors: HYTEG_EINVAL (null, dtype), HYTEG_ESTATE (level not refined). */
 int hyteg_autotune_choice(const hyteg_mesh* mesh, int level, int dtype, int* value);
 

@@ -80,7 +80,6 @@ Iface3<T> iface_of(const Mesh& m, const LevelDev& L) {
   f.n_items = L.n_ifi_ev;
   f.per_face = std::max(1, (L.n_face_pts + 31) / 32);
   f.n_pts = L.n_face_pts;
-  f.n_faces = L.n_face3;
   f.n_units = L.n_ifi_ev + f.per_face * L.n_face3;
   f.faces = L.face3;
   f.ab = L.face_ab;
@@ -235,7 +234,8 @@ template <class P, int MODE>
 cudaError_t launch_march(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
                          const ModeArgs* md, int count, cudaStream_t s, const March3Work* over) {
   const int n = ms[0]->levels[levels[0]].n;
-  if (n <= 128) return launch_march_s<P, MODE, 512>(ms, levels, xs, ys, md, count, s, over);
+  if constexpr (!std::is_same<P, ArF64Native>::value)  // native: the direct kernel up to there
+    if (n <= 128) return launch_march_s<P, MODE, 512>(ms, levels, xs, ys, md, count, s, over);
   if (n <= 512) return launch_march_s<P, MODE, 1280>(ms, levels, xs, ys, md, count, s, over);
   if constexpr (!P::kPoison) return launch_march_s<P, MODE, 4352>(ms, levels, xs, ys, md, count, s, over);
   return cudaErrorInvalidValue;
@@ -364,7 +364,6 @@ cudaError_t apply3d_prepare(int n) {
   if (n <= 128) {
     e = march_attr<ArF64FF, MODE_APPLY, 512>();
     if (e == cudaSuccess) e = march_attr<ArF32, MODE_APPLY, 512>();
-    if (e == cudaSuccess) e = march_attr<ArF64Native, MODE_APPLY, 512>();
   }
   return e;
 }

@@ -43,10 +43,10 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
     dev_free(m, x);
     dev_free(m, y);
   };
-  for (int dt = 1; dt <= 3 && err == cudaSuccess; ++dt) {
-    const std::array<int64_t, 4> key{m.device, m.n_cells, L.n, dt == 3 ? 1 : dt};
-    int best = dt == 3 ? L.z_chunks[1] : 0;
-    if (best == 0) {
+  for (int dt = 1; dt <= 2 && err == cudaSuccess; ++dt) {
+    const std::array<int64_t, 4> key{m.device, m.n_cells, L.n, dt};
+    int best = 0;
+    {
       std::lock_guard<std::mutex> lk(mu);
       auto it = cache.find(key);
       if (it != cache.end()) best = it->second;
@@ -105,6 +105,7 @@ cudaError_t march3d_autotune(Mesh& m, int level) {
     if ((err = set_march(m, L, dt, best)) != cudaSuccess) break;
     L.z_chunks[dt] = best;
   }
+  L.z_chunks[3] = L.z_chunks[1];
   if (err == cudaErrorMemoryAllocation) {  // no room for a list: the level keeps the one it has
     cudaGetLastError();
     err = cudaSuccess;

@@ -157,7 +157,7 @@ __device__ __forceinline__ void face3d_unit(const T* x, T* y, const Face3Rec* __
 template <class T>
 struct Iface3 {
   const IfItem* items;  // edges and vertices
-  int n_items, n_faces, per_face, n_pts, n_units;  // items, faces, units and points per face, units in all
+  int n_items, per_face, n_pts, n_units;  // items, units and points per face, units in all
   const Face3Rec* faces;
   const unsigned* ab;
   const Inc* incs;

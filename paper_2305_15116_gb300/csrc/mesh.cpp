@@ -618,7 +618,7 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     if (!L.direct3) {  // the columns' march (the autotuner may change the z-ranges)
       const cudaError_t ep = apply3d_prepare(n);
       if (ep != cudaSuccess) return std::string("cuda: ") + cudaGetErrorString(ep);
-      for (int dt = 1; dt <= 3; ++dt)
+      for (int dt = 1; dt <= (L.pts3 ? 2 : 3); ++dt)  // native fp64: the point table where there is one
         if (set_march(m, L, dt, std::max(2, n / 32)) != cudaSuccess) {
           cudaGetLastError();
           return "device allocation: 3D work list";

@@ -61,6 +61,11 @@ void fake_fail_malloc(long after, size_t bytes) {
 }
 int fake_malloc_armed() { return malloc_left >= 0; }
 void fake_fail_new(long after) { new_left = after; }
+int fake_has_kernel(const char* part, const char* and_part) {  // a kernel whose name holds both
+  for (const auto& n : names())
+    if (n.second.find(part) != std::string::npos && n.second.find(and_part) != std::string::npos) return 1;
+  return 0;
+}
 int fake_new_armed() { return new_left >= 0; }
 void fake_clear_log() { log_.clear(); }
 const char* fake_log() { return log_.c_str(); }  // kernel, device, grid, block, dynamic shared memory, cluster
