@@ -214,19 +214,22 @@ struct P2Ring {
 };
 constexpr int P2THREADS = 256;
 
-// The first blocks (per_cell for each macro) are p2_boundary_point's work.  A
-// macro's boundary points are few and wait on their gathers; beside the rows
-// that costs nothing.  Four launches as two (with k_p2_reduce): 421 -> 405 us
-// at level 10 with 32 macros (fp32 150 -> 135), 45 -> 26 us at level 7 with 24.
+// Some blocks of the launch are p2_boundary_point's work, a thread per point,
+// `stride` threads per macro.  A macro's boundary points are few and wait on
+// their gathers; beside the rows that costs nothing.  Four launches as two (with
+// k_p2_reduce): 421 -> 405 us at level 10 with 32 macros (fp32 150 -> 135), 45 ->
+// 26 us at level 7 with 24.
 template <class P>
 __global__ void __launch_bounds__(P2THREADS) k_p2_rows(const typename P::T* __restrict__ x, typename P::T* __restrict__ y,
                                                        const int4* __restrict__ tiles, int n_tiles, int64_t n_warps,
-                                                       Geo G, StencilPtr st, int n_points, int per_cell,
-                                                       int n_boundary) {
+                                                       Geo G, StencilPtr st, int n_points, int stride, int64_t n_cells,
+                                                       int first_boundary, int n_boundary) {
   pdl_trigger();
-  if ((int)blockIdx.x < n_boundary) {
-    const int cell = blockIdx.x / per_cell, i = (blockIdx.x - cell * per_cell) * P2THREADS + threadIdx.x;
-    if (i < n_points) p2_boundary_point<P>(x, y, G, st, cell, i);
+  const int bb = (int)blockIdx.x - first_boundary;
+  if (bb >= 0 && bb < n_boundary) {
+    const int64_t t = (int64_t)bb * P2THREADS + threadIdx.x, cell = t / stride;
+    const int i = int(t - cell * stride);
+    if (cell < n_cells && i < n_points) p2_boundary_point<P>(x, y, G, st, cell, i);
     return;
   }
   using T = typename P::T;
@@ -235,7 +238,7 @@ __global__ void __launch_bounds__(P2THREADS) k_p2_rows(const typename P::T* __re
   constexpr int P2RING = P2Ring<T>::value;
   __shared__ T ring_all[P2THREADS / 32][P2RING][4][32];
   __shared__ typename P::W wslice_all[P2THREADS / 32][REG ? 1 : 46];
-  const int64_t warp = ((int64_t)(blockIdx.x - n_boundary) * P2THREADS + threadIdx.x) >> 5;
+  const int64_t warp = ((int64_t)(bb < 0 ? (int)blockIdx.x : bb - n_boundary + first_boundary) * P2THREADS + threadIdx.x) >> 5;
   if (warp >= n_warps) return;  // whole warps leave together
   const int lane = threadIdx.x & 31;
   const int wid = threadIdx.x >> 5;
@@ -523,12 +526,24 @@ cudaError_t launch_t(const Mesh& m, const LevelDev& L, const void* x, void* y, c
   StencilPtr st{L.p2_st64, L.p2_st32, L.p2_hi, L.p2_lo};
   *what = "P2 row kernel";
   const int64_t n_warps = (int64_t)L.n_p2_tiles * m.n_cells;
-  const int nb = L.n == 1 ? 3 : 4 * L.n - 2, per_cell = (nb + P2THREADS - 1) / P2THREADS;
-  const int64_t n_boundary = (int64_t)per_cell * m.n_cells;
+  const int nb = L.n == 1 ? 3 : 4 * L.n - 2;
+  // From n = 64 on the 4n - 2 boundary points of a macro fill whole blocks but for
+  // two, and a warp's points lie on one side (level 6, 2048 macros: float-float 251
+  // us, 271 without a gap between the macros); below, the macros follow one
+  // another without a gap (20000 macros at level 1: 608 -> 94 us, 2048 at level 5:
+  // 123 -> 112).
+  const int stride = L.n >= 64 ? (nb + P2THREADS - 1) / P2THREADS * P2THREADS : nb;
+  const int64_t n_boundary = (stride * m.n_cells + P2THREADS - 1) / P2THREADS;
   const int64_t blocks = n_boundary + (n_warps * 32 + P2THREADS - 1) / P2THREADS;
   if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  // Native fp64's rows wait for the fp64 pipe: on low levels they start first
+  // (level 6, 128 macros 41 against 66 us with the boundary first, level 5, 2048
+  // macros 167 against 191; from level 7 on the same, or slower: level 8, 32 macros
+  // 141 against 109).
+  const bool last = std::is_same<P, ArF64Native>::value && L.n < 128;
   k_p2_rows<P><<<(unsigned)blocks, P2THREADS, 0, s>>>((const T*)x, (T*)y, L.p2_tiles, L.n_p2_tiles, n_warps, G, st, nb,
-                                                      per_cell, (int)n_boundary);
+                                                      stride, m.n_cells, last ? (int)(blocks - n_boundary) : 0,
+                                                      (int)n_boundary);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (ev_mid && (e = cudaEventRecord(ev_mid, s)) != cudaSuccess) return e;
