@@ -73,8 +73,8 @@ extern "C" {
                                 float-float range (zero or 2^-80 <= |x| < 2^64)
                                 are recomputed with native fp64 FMAs in the same
                                 launch, and levels with a stencil whose largest
-                                weight leaves 2^-20 .. 2^14, and 3D levels
-                                above 9, run the native kernels */
+                                weight leaves 2^-20 .. 2^14 run the native
+                                kernels */
 #define HYTEG_F32       2    /* float32 vectors, fp32 FMA arithmetic */
 #define HYTEG_F64_IEEE  3    /* float64 vectors, native fp64 FMA arithmetic */
 

@@ -15,6 +15,7 @@
 #include "direct.cuh"
 #include "march3d.cuh"
 #include "per_device.h"
+#include "rows3d.cuh"
 
 namespace hyteg {
 
@@ -228,39 +229,68 @@ cudaError_t launch_march_s(const Mesh* const* ms, const int* levels, const void*
 }
 
 // The slot size is a constant of the kernel: the columns of a block with their
-// neighbour rows, 256 + 2n, for n up to 128, 512 and 2048 (float-float up to
-// 512, LevelDev::ff_ok).
+// neighbour rows, 256 + 2n, for n up to 128; native fp64, which has the point table
+// up to there, for level 8.
 template <class P, int MODE>
 cudaError_t launch_march(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
                          const ModeArgs* md, int count, cudaStream_t s, const March3Work* over) {
-  const int n = ms[0]->levels[levels[0]].n;
-  if constexpr (!std::is_same<P, ArF64Native>::value)  // native: the direct kernel up to there
-    if (n <= 128) return launch_march_s<P, MODE, 512>(ms, levels, xs, ys, md, count, s, over);
-  if (n <= 512) return launch_march_s<P, MODE, 1280>(ms, levels, xs, ys, md, count, s, over);
-  if constexpr (!P::kPoison) return launch_march_s<P, MODE, 4352>(ms, levels, xs, ys, md, count, s, over);
-  return cudaErrorInvalidValue;
+  return launch_march_s<P, MODE, std::is_same<P, ArF64Native>::value ? 1280 : 512>(ms, levels, xs, ys, md, count, s,
+                                                                                   over);
+}
+
+template <class P, int MODE>
+cudaError_t launch_rows(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
+                        const ModeArgs* md, int count, cudaStream_t s) {
+  using B = Rows3<P, MODE>;
+  using T = typename P::T;
+  for (int i = 0; i < count; ++i) {  // such levels fill the device each by itself
+    const Mesh& m = *ms[i];
+    const LevelDev& L = m.levels[levels[i]];
+    typename B::Prm p;
+    p.x = static_cast<const T*>(xs[i]);
+    p.y = static_cast<T*>(ys[i]);
+    p.tiles = L.tiles3;
+    p.n_tiles = L.n_tiles3;
+    p.n_warps = int64_t(L.n_tiles3) * m.n_cells;
+    p.f = iface_of<T>(m, L);
+    p.st = StencilPtr{L.st64, L.st32, L.st_hi, L.st_lo};
+    p.md = md ? md[i] : ModeArgs{nullptr, nullptr, 0.0};
+    p.n = L.n;
+    p.S = L.slots_per_macro;
+    p.n_if_blocks = (p.f.n_units + B::kThreads / 32 - 1) / (B::kThreads / 32);
+    const int64_t blocks = p.n_if_blocks + (p.n_warps * 32 + B::kThreads - 1) / B::kThreads;
+    if (L.n_tiles3 == 0 || blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    const cudaError_t e = launch_one<B>(p, int(blocks), s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // The members whose vectors are small take the direct kernel, the others the
-// march; each kind shares its launches.
+// march or the rows (takes_rows3); each kind shares its launches.
 template <class P, int MODE>
 cudaError_t launch_t(const Mesh* const* ms, const int* levels, const void* const* xs, void* const* ys,
                      const ModeArgs* md, int count, cudaStream_t s) {
   // native fp64 is bound by the fp64 pipe either way, and the direct kernel's
   // occupancy suits it better (level 6, 384 macro-tets: 488 against 600 us)
   constexpr bool native = std::is_same<P, ArF64Native>::value;
-  auto takes_direct = [](const LevelDev& L) { return L.direct3 || (native && L.pts3); };
-  if (count == 1)
-    return takes_direct(ms[0]->levels[levels[0]]) ? launch_direct<P, MODE>(ms, levels, xs, ys, md, 1, s)
-                                                  : launch_march<P, MODE>(ms, levels, xs, ys, md, 1, s, nullptr);
-  for (int direct = 0; direct < 2; ++direct) {
+  constexpr int dt = sizeof(typename P::T) == 4 ? 2 : (native ? 3 : 1);
+  auto kind = [](const LevelDev& L) { return L.direct3 || (native && L.pts3) ? 0 : L.rows3[dt] ? 2 : 1; };
+  auto go = [&](int k, const Mesh* const* m, const int* l, const void* const* x, void* const* y, const ModeArgs* a,
+                int cnt) {
+    return k == 0   ? launch_direct<P, MODE>(m, l, x, y, a, cnt, s)
+           : k == 1 ? launch_march<P, MODE>(m, l, x, y, a, cnt, s, nullptr)
+                    : launch_rows<P, MODE>(m, l, x, y, a, cnt, s);
+  };
+  if (count == 1) return go(kind(ms[0]->levels[levels[0]]), ms, levels, xs, ys, md, 1);
+  for (int k = 0; k < 3; ++k) {
     std::vector<const Mesh*> mm;
     std::vector<int> lv;
     std::vector<const void*> xx;
     std::vector<void*> yy;
     std::vector<ModeArgs> mo;
     for (int i = 0; i < count; ++i) {
-      if (int(takes_direct(ms[i]->levels[levels[i]])) != direct) continue;
+      if (kind(ms[i]->levels[levels[i]]) != k) continue;
       mm.push_back(ms[i]);
       lv.push_back(levels[i]);
       xx.push_back(xs[i]);
@@ -268,11 +298,7 @@ cudaError_t launch_t(const Mesh* const* ms, const int* levels, const void* const
       if (md) mo.push_back(md[i]);
     }
     if (mm.empty()) continue;
-    const int k = int(mm.size());
-    const ModeArgs* mp = md ? mo.data() : nullptr;
-    const cudaError_t e =
-        direct ? launch_direct<P, MODE>(mm.data(), lv.data(), xx.data(), yy.data(), mp, k, s)
-               : launch_march<P, MODE>(mm.data(), lv.data(), xx.data(), yy.data(), mp, k, s, nullptr);
+    const cudaError_t e = go(k, mm.data(), lv.data(), xx.data(), yy.data(), md ? mo.data() : nullptr, int(mm.size()));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -360,12 +386,34 @@ cudaError_t launch_sum_copies3d(const Mesh* const* ms, const int* levels, const 
 }
 
 cudaError_t apply3d_prepare(int n) {
-  cudaError_t e = cudaSuccess;
-  if (n <= 128) {
-    e = march_attr<ArF64FF, MODE_APPLY, 512>();
-    if (e == cudaSuccess) e = march_attr<ArF32, MODE_APPLY, 512>();
+  if (n > 128) return cudaSuccess;
+  const cudaError_t e = march_attr<ArF64FF, MODE_APPLY, 512>();
+  return e == cudaSuccess ? march_attr<ArF32, MODE_APPLY, 512>() : e;
+}
+
+// us per apply, rows / march: float-float and fp32 on level 8, 1 macro 45 / 90 and
+// 15 / 29, 6 macros 228 / 264 and 69 / 113, 48 macros 1804 / 2133 and 556 / 953; on
+// level 7, 5 macros 41 / 46 and 15 / 18, 9 macros 62 / 46 and 20 / 18.  Native fp64
+// on level 8, even numbers of macros 595 / 546 (6), odd ones, whose last pair of
+// the march is half empty, 119 / 202 (1), 499 / 544 (5), 1457 / 1456 (15); on level
+// 9, 6 macros 4228 / 4242.
+bool takes_rows3(int n, int64_t n_cells, int dt) {
+  if (dt == 3) return n >= 512 || (n >= 256 && n_cells % 2 && n_cells < 16);
+  return n >= 256 || (n >= 128 && slots_per_macro(3, 7) * n_cells <= kRows3Slots);
+}
+
+std::vector<int4> tile_list_rows3(int n) {
+  // chunks of 32 rows (level 7, 384 macro-tets: 3.94 -> 3.50 ms float-float and
+  // 1.16 -> 1.11 ms fp32 against 64; a warp walks its rows serially)
+  constexpr int kRows = 32;
+  std::vector<int4> t;
+  for (int z = 1; z <= n - 3; ++z) {
+    const int M = n + 1 - z;
+    for (int x0 = 1; x0 <= M - 3; x0 += ROWS3_WIDTH)
+      for (int y0 = 1; y0 <= M - 2 - x0; y0 += kRows)
+        t.push_back(make_int4(x0, y0, std::min(y0 + kRows, M - 1 - x0), z));
   }
-  return e;
+  return t;
 }
 
 void march3d_lists(int n, int chunks, int dtype, std::vector<int4>& work, int& stride) {

@@ -103,6 +103,11 @@ struct LevelDev {
   // fp64): the columns' march, and the z-ranges per macro that the autotuner
   // picked for it (0: not tuned, two ranges)
   March3Work march[4];
+  // the element types whose products walk along rows instead (rows3d.cuh), and
+  // that kernel's tiles (x0, y0, y1, z) of a macro
+  bool rows3[4] = {false, false, false, false};
+  int4* tiles3 = nullptr;
+  int n_tiles3 = 0;
   int z_chunks[4] = {0, 0, 0, 0};
   // host copy of the class stencils (multigrid set-up)
   std::vector<double> st_host;
@@ -270,6 +275,9 @@ std::string build_level(Mesh& m, int level, LevelDev& out);
 // z-ranges (-, z0, z1, -): a macro cut into `chunks` ranges of about equal
 // slice counts
 std::vector<int4> z_ranges(int n, int chunks);
+// whether a level's 3D products of element type dt walk along rows, and the tiles
+bool takes_rows3(int n, int64_t n_cells, int dt);
+std::vector<int4> tile_list_rows3(int n);
 // the work list of the 3D march for `chunks` z-ranges; on the device (`out` only
 // if that succeeds), and as the level's list in place of the one it had (which
 // stays if that fails)
@@ -381,11 +389,14 @@ cudaError_t launch_sweep2d_group(bool jacobi, const Mesh* const* ms, const int* 
 constexpr int64_t kDirect2MaxSlots = 3 * (int64_t(1) << 17);
 // the finest level of 3D products (32-bit slots inside a macro)
 constexpr int kMaxProductLevel3 = 11;
-// Levels whose vectors the direct 3D kernel takes (LevelDev::direct3), and the
-// levels with its point table (which native fp64 always uses).
-constexpr int kDirect3MaxN = 64;
+// Vectors that the direct 3D kernel takes (LevelDev::direct3; levels 0 to 3 at any
+// size), and the levels with its point table (which native fp64 always uses).  Level
+// 7, us per apply, direct / rows: 1 macro float-float 7.3 / 21.9, fp32 4.3 / 13.1; 2
+// macros 13.3 / 23.8, 4.9 / 10.3.
 constexpr int64_t kDirect3MaxSlots = int64_t(1) << 20;
 constexpr int kDirect3TableN = 128;
+// level 7: vectors that walk along rows rather than march (takes_rows3)
+constexpr int64_t kRows3Slots = int64_t(1) << 21;
 // the 3D apply of several meshes, one launch per kernel kind, interface step
 // included (partial: every interface copy keeps its own macro's partial row)
 cudaError_t launch_apply3d_group(int dtype, bool partial, const Mesh* const* ms, const int* levels,

@@ -173,10 +173,10 @@ struct March3 {
   static constexpr int kThreads = MARCH_COLS;
   static constexpr bool kLateWait = true;  // the tables first
   // slices in the ring; float-float: split slices kept, from which the values
-  // "below" are read again (32 registers fewer, three blocks per SM)
-  static constexpr int kPlanes = kSplit ? (STRIDE <= 512 ? 4 : 3) : 0;
-  static constexpr bool kReread = kPlanes == 4;
-  static constexpr int kDepth = kReread ? 4 : sizeof(T) == 4 && STRIDE <= 512 ? 6 : 3;
+  // "below" are read again (32 registers fewer)
+  static constexpr int kPlanes = kSplit ? 4 : 0;
+  static constexpr bool kReread = kSplit;
+  static constexpr int kDepth = kReread ? 4 : sizeof(T) == 4 ? 6 : 3;
   // fp32: three blocks per SM.  At four the 64 registers spill around the
   // interface step and in the marching (level 7, 72 macro-tets: 105 against 94 us).
   static constexpr int kMinBlocks = STRIDE > 512 ? 1 : sizeof(T) == 4 ? 3 : 2;
@@ -438,8 +438,8 @@ struct March3 {
         stage(std::integral_constant<int, 4>{});
       } else if constexpr (kSplit) {
         stage(std::integral_constant<int, 2>{});
+        stage(std::integral_constant<int, 3>{});
       }
-      if constexpr (kReread) stage(std::integral_constant<int, 3>{});
     }
     // While the first slices land: this block's share of the interface step, in
     // the order of the macros.  (Interface blocks between the marching ones

@@ -337,6 +337,7 @@ void free_level(const Mesh& m, LevelDev& L) {
   dev_free(m, L.items);
   for (int t = 0; t < 4; ++t) dev_free(m, L.march[t].work);
   dev_free(m, L.pts3);
+  dev_free(m, L.tiles3);
   dev_free(m, L.ifi);
   dev_free(m, L.face3);
   dev_free(m, L.face_ab);
@@ -477,9 +478,7 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     sth[i] = float(ws);
     stl[i] = float(ws - double(sth[i]));
   }
-  // a slice's columns with their neighbour rows, split for the 3D march, fit
-  // in shared memory up to n = 512; above, native fp64
-  L.ff_ok = ff_weights_in_range(st, ncls * nw) && (d == 2 || n <= 512);
+  L.ff_ok = ff_weights_in_range(st, ncls * nw);
 
   // ---- 2D macro-interior work lists: strips of columns x chunks of rows ----
   // a warp loads 64 consecutive columns and writes the 62 inner ones.  A warp
@@ -601,7 +600,7 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     std::vector<float> wf_f(wf.begin(), wf.end());
     if (!(err = upload(m, &L.wf64, wf)).empty()) return err;
     if (!(err = upload(m, &L.wf32, wf_f)).empty()) return err;
-    L.direct3 = n <= 8 || (n <= kDirect3MaxN && L.slots_per_macro * m.n_cells <= kDirect3MaxSlots);
+    L.direct3 = n <= 8 || L.slots_per_macro * m.n_cells <= kDirect3MaxSlots;  // n <= 128
     if (n <= kDirect3TableN) {  // the macro-interior points in slot order: (slot, A | M << 16)
       std::vector<int2> pts;
       int slot = 0;
@@ -618,11 +617,19 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     if (!L.direct3) {  // the columns' march (the autotuner may change the z-ranges)
       const cudaError_t ep = apply3d_prepare(n);
       if (ep != cudaSuccess) return std::string("cuda: ") + cudaGetErrorString(ep);
-      for (int dt = 1; dt <= (L.pts3 ? 2 : 3); ++dt)  // native fp64: the point table where there is one
+      for (int dt = 1; dt <= (L.pts3 ? 2 : 3); ++dt) {  // native fp64: the point table where there is one
+        L.rows3[dt] = takes_rows3(n, m.n_cells, dt);
+        if (L.rows3[dt]) continue;
         if (set_march(m, L, dt, std::max(2, n / 32)) != cudaSuccess) {
           cudaGetLastError();
           return "device allocation: 3D work list";
         }
+      }
+      if (L.rows3[1] || L.rows3[2] || L.rows3[3]) {
+        const std::vector<int4> t = tile_list_rows3(n);
+        L.n_tiles3 = int(t.size());
+        if (!(err = upload(m, &L.tiles3, t)).empty()) return err;
+      }
     }
   }
   if (d == 2) return build_p2_level(m, level, L);

@@ -18,18 +18,17 @@ def test_level_12_is_refused_as_an_argument():
 
 
 def test_native_fp64_marches_above_its_point_table_only():
-    """Up to level 7 native products take the point table: no march kernel and no
-    work lists are built for them there."""
+    """Up to level 7 native products take the point table: there is no march kernel
+    for them."""
     out = fake_cuda.run("""
     m = unit_cube_kuhn_mesh(2, 0.1, 0)
     M = H.Mesh(m.coords, m.cells).refine(5)
-    lists = []
+    marched = []
     for level in (6, 7, 8):
-        n = F.fake_uploads()
         M.refine(level)
         clear()
         apply(M, level, H.F64_IEEE)
-        lists.append((F.fake_uploads() - n, "March3" in launches()[0]["name"]))
-    print(lists[1][0] == lists[2][0], [l[1] for l in lists], F.fake_has_kernel(b"March3INS_11ArF64Native", b"Li512E"))
+        marched.append("March3" in launches()[0]["name"])
+    print(marched, F.fake_has_kernel(b"March3INS_11ArF64Native", b"Li512E"))
     """)
-    assert out == ["True [False, False, True] 0"]
+    assert out == ["[False, False, True] 0"]

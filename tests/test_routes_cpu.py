@@ -22,3 +22,36 @@ def test_p2_boundary_points_share_blocks(k, level):
         print(rows["grid"] * rows["block"] <= 2 * len(m.cells) * (points + 32 * tiles) + 512)
     """)
     assert out == ["True"] * 3
+
+
+@pytest.mark.parametrize("count", [1, 2, 3, 6, 48])
+def test_kernel_of_a_3d_level(count):
+    """A thread per point for at most 2^20 slots (native fp64 up to level 7), rows for
+    fine levels, the march between them."""
+    out = fake_cuda.run(f"""
+    m = unit_cube_kuhn_mesh(2, 0.1, 0)
+    used, cells = np.unique(m.cells[:{count}], return_inverse=True)
+    M = H.Mesh(m.coords[used], cells.reshape(-1, 4)).refine(9)
+    for level in (5, 6, 7, 8, 9):
+        r = []
+        for dtype in (H.F64, H.F32, H.F64_IEEE):
+            clear()
+            assert apply(M, level, dtype) == 0
+            l, = launches()
+            r.append([k for k in ("Direct3", "March3", "Rows3") if k in l["name"]][0][0])
+        print("".join(r))
+    """)
+    march6, march7 = count >= 22, count >= 6
+    seven = "DDD" if count <= 2 else "MMD" if march7 else "RRD"
+    assert out == ["MMD" if count >= 162 else "DDD", "MMD" if march6 else "DDD", seven,
+                   "RRR" if count % 2 else "RRM", "RRR"]
+
+
+def test_fused_sweeps_of_fine_3d_levels():
+    out = fake_cuda.run("""
+    M = H.Mesh(np.eye(4)[:, :3], np.arange(4)[None]).refine(8).solver_setup(8)
+    clear()
+    print(C.lib.hyteg_vcycle(M._h, 8, H.F32, X, Y, None), sum("Rows3" in l["name"] for l in launches()),
+          any("Jacobi" in l["name"] for l in launches()))
+    """)
+    assert out == ["0 7 False"]
