@@ -2,10 +2,9 @@
 // per mesh runs every phase of the cycle from level `top` down to the direct
 // solve on level 0 and back up, a cluster barrier between the phases.
 //
-// On these levels a phase is a few microseconds of launch, table loads and one
-// round of gathers for well under a microsecond of work, and a cycle has eight
-// phases per level (one V-cycle on 24 macro-triangles at level 6: 55 launches,
-// 199 us).  In the cluster a phase costs its gathers and one hardware barrier.
+// On these levels a phase is a launch, table loads and one round of gathers for well
+// under a microsecond of work, and a cycle has eight phases per level.  In the
+// cluster a phase costs its gathers and one hardware barrier.
 //
 // The vectors stay in global memory (L2): every load of a vector goes to L2
 // (ld.cg), since other blocks of the cluster write it between barriers, whose
@@ -13,11 +12,19 @@
 // launches, point by point (direct.cuh, lattice.cuh, transfer.cuh), so a cycle
 // gives the same bits.
 //
-// Measured: that cycle 188 -> 128 us; a V-cycle on 32 macro-triangles at level
-// 10 781 -> 730 us; a level-8 solve 6.01 -> 4.86 ms.  384 threads per block
-// (1024 spilled: 156 us; 256: 131, 128: 150), 16 blocks (8: 142 us).  In 3D the
-// launches stay: the gathers are twice as long and need the whole device (a
-// level-5 solve 5.44 against 6.21 ms).
+// Which levels (solver_setup): those that give every warp of the cluster at most
+// one task of a phase, an interface item or 32 interior points, from level 1 up,
+// and level 0 with at most a slot per thread.  A second round of tasks costs a
+// phase's chain of loads again, while a launch spreads them over the device.  A
+// cycle in us, all levels in launches / this rule / one task more per warp and so
+// on up to 32768 slots: 2 macros level 4 68 / 52 / 52, level 7 109 / 98 / 106; 18
+// macros level 4 67 / 63 / 63, level 5 81 / 79 / 85; 50 macros level 5 85 / 84 / 106;
+// 128 macros level 4 72 / 73 / 122; 512 macros level 3 69 / 69 / 203; 2048 macros
+// level 0 52 / 45 / 45 and level 2 104 / 95 / 437.
+//
+// 384 threads per block (1024 spilled: 156 us for a cycle of 128; 256: 131, 128:
+// 150), 16 blocks (8: 142 us).  In 3D the launches stay: the gathers are twice as
+// long and need the whole device (a level-5 solve 5.44 against 6.21 ms).
 #include <vector>
 
 #include "direct.cuh"
@@ -126,28 +133,25 @@ struct Cycle {
   __device__ __forceinline__ void copy(float* dst, const float* src, int total) const {
     for (int i = gw * 32 + lane; i < total; i += nw * 32) dst[i] = src ? __ldcg(src + i) : 0.0f;
   }
-  // level 0: u = A0^{-1} b on the coarse vertices, written to every copy; the
-  // right-hand side staged by every block, the sum over the vertices in order
+  // level 0: u = A0^{-1} b on the coarse vertices, written to every copy, a thread
+  // per slot; the right-hand side staged by every block, the sum over the vertices
+  // in order
   __device__ __forceinline__ void level0(const float* b, float* u, float* sh) const {
-    const int ns = p.n_cells * 3;
+    const int s = gw * 32 + lane;
+    const bool live = s < p.n_cells * 3;
+    const float* __restrict__ row = p.a0inv + (int64_t)(live ? __ldg(p.v_of_slot + s) : 0) * p.V;
     float acc = 0.0f;
-    const int first = gw * 32 + lane, stride = nw * 32;
-    for (int s0 = 0; s0 < ns; s0 += stride) {  // every thread of the cluster in step
-      const int s = s0 + first;
-      const float* __restrict__ row = p.a0inv + (int64_t)(s < ns ? __ldg(p.v_of_slot + s) : 0) * p.V;
-      acc = 0.0f;
-      for (int j0 = 0; j0 < p.V; j0 += CTHREADS) {
-        const int cnt = min(CTHREADS, p.V - j0);
-        __syncthreads();
-        if ((int)threadIdx.x < cnt) sh[threadIdx.x] = __ldcg(b + __ldg(p.slot_of_v + j0 + threadIdx.x));
-        __syncthreads();
-        if (s < ns) {
+    for (int j0 = 0; j0 < p.V; j0 += CTHREADS) {
+      const int cnt = min(CTHREADS, p.V - j0);
+      __syncthreads();
+      if ((int)threadIdx.x < cnt) sh[threadIdx.x] = __ldcg(b + __ldg(p.slot_of_v + j0 + threadIdx.x));
+      __syncthreads();
+      if (live) {
 #pragma unroll 8
-          for (int j = 0; j < cnt; ++j) acc = __fmaf_rn(__ldg(row + j0 + j), sh[j], acc);
-        }
+        for (int j = 0; j < cnt; ++j) acc = __fmaf_rn(__ldg(row + j0 + j), sh[j], acc);
       }
-      if (s < ns) u[s] = acc;
     }
+    if (live) u[s] = acc;
   }
 };
 
@@ -263,9 +267,11 @@ cudaError_t launch_coarse_cycle(Mesh* const* ms, int cnt, int l, const float* co
   return cudaSuccess;
 }
 
-cudaError_t coarse_cycle_prepare() {
+cudaError_t coarse_cycle_prepare(int* warps) {
   int size = 0;
-  return cluster_size(&size);
+  const cudaError_t e = cluster_size(&size);
+  *warps = size * (CTHREADS / 32);
+  return e;
 }
 
 }  // namespace hyteg

@@ -350,11 +350,8 @@ void solver_free(Mesh& m);
 // one launch, l <= Solver::coarse_top (coarse.cu); vectors as vcycle_g.
 cudaError_t launch_coarse_cycle(Mesh* const* ms, int cnt, int l, const float* const* b, float* const* u,
                                 bool first_done, cudaStream_t s);
-cudaError_t coarse_cycle_prepare();  // before any stream capture
-// 2D levels of at most so many slots (one V-cycle on 32 macro-triangles at level
-// 10: 781 us without, 757, 734 and 723 us with a limit of 4000, 16000 and 32000
-// slots; with 1024 threads per block 64000 was 10 % slower than 32000)
-constexpr int64_t kCoarseMaxSlots = 32768;
+// finds the cluster on the current device (before any stream capture): its warps
+cudaError_t coarse_cycle_prepare(int* warps);
 // inverse diagonals (fp64, fp32) and owner flags of one level, on the device
 cudaError_t mg_diag_setup(const Mesh& m, int level, MgLevel& g, cudaStream_t s);
 cudaError_t mg_restrict(const Mesh& m, int fine_level, int dtype, const void* rf, void* bc, cudaStream_t s);

@@ -475,20 +475,24 @@ std::string solver_setup(Mesh& m, int max_level, int nu1, int nu2, double omega)
   if (!(err = alloc_vec(m, &sv.red, size_t(1024 + 8))).empty()) return err;
   // the levels of the coarse-cycle kernel
   std::vector<CoarseLev> cl;
-  for (int l = 0; d == 2 && l <= max_level; ++l) {
-    const LevelDev& L = m.levels[l];
-    if (L.slots_per_macro * m.n_cells > kCoarseMaxSlots) break;
-    const MgLevel& g = sv.lv[l];
-    const int n = L.n;
-    cl.push_back({g.u32, g.b32, g.y32, g.r32, g.dinv32, g.multinv32, L.st32, g.lpts, L.ifi, L.n_ifi,
-                  n > 2 ? (n - 1) * (n - 2) / 2 : 0, n, int(L.slots_per_macro)});
-    sv.coarse_top = l;
-  }
-  if (!cl.empty()) {
-    if (!(err = upload_vec(m, &sv.coarse, cl)).empty()) return err;
-    const cudaError_t ep = coarse_cycle_prepare();
+  int warps = 0;
+  if (d == 2) {
+    const cudaError_t ep = coarse_cycle_prepare(&warps);
     if (ep != cudaSuccess) return std::string("cuda: ") + cudaGetErrorString(ep);
   }
+  for (int l = 0; d == 2 && l <= max_level; ++l) {
+    const LevelDev& L = m.levels[l];
+    const int n = L.n, n_inner = n > 2 ? (n - 1) * (n - 2) / 2 : 0;
+    // tasks of a phase, in warps (coarse.cu)
+    const int64_t tasks = l == 0 ? (L.slots_per_macro * m.n_cells + 31) / 32
+                                 : L.n_ifi + m.n_cells * ((n_inner + 31) / 32);
+    if (tasks > warps) break;
+    const MgLevel& g = sv.lv[l];
+    cl.push_back({g.u32, g.b32, g.y32, g.r32, g.dinv32, g.multinv32, L.st32, g.lpts, L.ifi, L.n_ifi, n_inner, n,
+                  int(L.slots_per_macro)});
+    sv.coarse_top = l;
+  }
+  if (!cl.empty() && !(err = upload_vec(m, &sv.coarse, cl)).empty()) return err;
   const cudaError_t e = dev_sync(m);
   if (e != cudaSuccess) return std::string("cuda: set-up: ") + cudaGetErrorString(e);
   return "";

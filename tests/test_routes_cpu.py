@@ -55,3 +55,41 @@ def test_fused_sweeps_of_fine_3d_levels():
           any("Jacobi" in l["name"] for l in launches()))
     """)
     assert out == ["0 7 False"]
+
+
+@pytest.mark.parametrize("k,level", [(1, 7), (2, 5), (5, 5), (8, 1), (32, 1), (45, 2)])
+def test_coarse_levels_of_a_cycle(k, level):
+    """The coarse levels' kernel takes the levels that give each of its 192 warps at
+    most one task of a phase (level 0: 32 slots), the others are launches."""
+    out = fake_cuda.run(f"""
+    m = unit_square_mesh({k}, 0.1, 0)
+    M = H.Mesh(m.coords, m.cells).refine({level}).solver_setup({level})
+    clear()
+    assert C.lib.hyteg_vcycle(M._h, {level}, H.F32, X, Y, None) == 0
+    coarse = [l["cluster"] for l in launches() if "k_coarse" in l["name"]]
+    top, cells = -1, len(m.cells)
+    V, E = ({k} + 1) ** 2, 3 * {k} ** 2 + 2 * {k}
+    for l in range({level} + 1):
+        n = 2 ** l
+        tasks = (3 * cells + 31) // 32 if l == 0 else V + E * ((n - 1 + 31) // 32) + cells * (((n - 1) * (n - 2) // 2 + 31) // 32)
+        if tasks > 192:
+            break
+        top = l
+    # a launch per phase above: two more pre-sweeps (three on the finest level), the
+    # residual, both transfers, three sweeps; the level-0 solve where it is a launch
+    n = sum(8 + (l == {level}) for l in range(1, {level} + 1) if l > top) + 1
+    print(coarse == ([16] if top >= 0 else []), len(launches()) == n, top)
+    """)
+    assert out[0].startswith("True True"), out
+
+
+@pytest.mark.parametrize("k", [1, 3])
+def test_no_second_round_in_the_coarse_levels(k):
+    out = fake_cuda.run(f"""
+    m = unit_square_mesh(24, 0.1, 0)
+    M = H.Mesh(m.coords, m.cells).refine({k}).solver_setup({k})
+    clear()
+    C.lib.hyteg_vcycle(M._h, {k}, H.F32, X, Y, None)
+    print(len(launches()) > 8 * {k})
+    """)
+    assert out == ["True"]
