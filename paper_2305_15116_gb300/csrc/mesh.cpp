@@ -498,7 +498,7 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
   }
   auto strips = [&](int th_max, int width) {
     std::vector<int4> tl;
-    if (d != 2) return tl;
+    if (d != 2 || L.slots_per_macro * m.n_cells <= kDirect2MaxSlots) return tl;  // not walked
     auto n_warps = [&](int th) {
       int64_t w = 0;
       for (int x0 = 1; x0 <= n - 2; x0 += width) w += (n - 1 - x0 + th - 1) / th;
@@ -602,15 +602,13 @@ std::string build_level(Mesh& m, int level, LevelDev& L) {
     if (!(err = upload(m, &L.wf32, wf_f)).empty()) return err;
     L.direct3 = n <= 8 || L.slots_per_macro * m.n_cells <= kDirect3MaxSlots;  // n <= 128
     if (n <= kDirect3TableN) {  // the macro-interior points in slot order: (slot, A | M << 16)
-      std::vector<int2> pts;
-      int slot = 0;
+      std::vector<int2> pts(n > 3 ? size_t(n - 1) * (n - 2) * (n - 3) / 6 : 0);
+      int2* p = pts.data();
+      int row = 0;  // slot of the row's first point
       for (int z = 0; z <= n; ++z)
-        for (int y = 0; y <= n - z; ++y)
-          for (int x = 0; x <= n - z - y; ++x, ++slot)
-            if (x > 0 && y > 0 && z > 0 && x + y + z < n) {
-              const int M = n + 1 - z;
-              pts.push_back(make_int2(slot, (M - y) | (M << 16)));
-            }
+        for (int y = 0, M = n + 1 - z; y < M; row += M - y, ++y)
+          if (y > 0 && z > 0)
+            for (int x = 1; x + 1 < M - y; ++x) *p++ = make_int2(row + x, (M - y) | (M << 16));
       L.n_pts3 = int(pts.size());
       if (!(err = upload(m, &L.pts3, pts)).empty()) return err;
     }

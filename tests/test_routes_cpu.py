@@ -93,3 +93,23 @@ def test_no_second_round_in_the_coarse_levels(k):
     print(len(launches()) > 8 * {k})
     """)
     assert out == ["True"]
+
+
+def test_no_tiles_for_levels_that_are_not_walked():
+    """A 2D level whose products take a thread per point is refined without the
+    walker's two tile lists."""
+    out = fake_cuda.run("""
+    from inputs import rect_mesh
+    m = rect_mesh(3, 1, 0.1, 0)
+    M = H.Mesh(m.coords, m.cells).refine(7)
+    n = []
+    for level in (8, 9):  # 199 k and 791 k slots
+        a = F.fake_uploads()
+        M.refine(level)
+        n.append(F.fake_uploads() - a)
+        clear()
+        apply(M, level)
+        n.append("Direct2" in launches()[0]["name"])
+    print(n[2] - n[0], n[1], n[3])
+    """)
+    assert out == ["2 True False"]
