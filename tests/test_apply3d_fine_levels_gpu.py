@@ -55,3 +55,36 @@ def test_every_slot(cuda, L, count):
                                               ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)), "partial")
             assert torch.equal(p, want)
     M.close()
+
+
+@pytest.mark.parametrize("odd", [0.0, 1e-4])
+@pytest.mark.parametrize("kind,L,count", [("f64_ieee", 8, 2), ("f64_ieee", 8, 4), ("f64", 7, 6), ("f32", 7, 6),
+                                          ("f64", 7, 3), ("f32", 7, 3), ("f64", 8, 2)])
+def test_a_macro_alone_has_the_same_bits(cuda, kind, L, count, odd):
+    """Marched (native fp64 on level 8, six macros on level 7) or walked along rows in
+    a mesh, a macro's partial rows are those of the macro alone, which takes rows or a
+    thread per point."""
+    import torch
+    import paper_2305_15116_gb300 as H
+    from paper_2305_15116_gb300 import _capi as C
+    coords, cells = _macros(count)
+    code = {"f64": H.F64, "f32": H.F32, "f64_ieee": H.F64_IEEE}[kind]
+
+    def partial(M, x):
+        y = torch.full_like(x, float("nan"))
+        C.check(C.lib.hyteg_apply_partial(M._h, L, code, x.data_ptr(), y.data_ptr(),
+                                          ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)), "partial")
+        return y
+    M = H.Mesh(coords, cells, bc=H.BC_NONE).refine(L)
+    ns, _ = M.num_slots(L)
+    S = ns // count
+    g = torch.Generator(device="cuda").manual_seed(count)
+    x = torch.rand(ns, generator=g, device="cuda", dtype=torch.float64) * 2 - 1
+    pick = torch.rand(ns, generator=g, device="cuda") < odd  # outside the float-float range, inside fp32's
+    x = torch.where(pick, x * 1e-30, x).to(torch.float32 if kind == "f32" else torch.float64)
+    y = partial(M, x)
+    for c in (0, count - 1):
+        One = H.Mesh(coords[cells[c]], np.arange(4)[None], bc=H.BC_NONE).refine(L)
+        assert torch.equal(partial(One, x[c * S:(c + 1) * S].clone()), y[c * S:(c + 1) * S]), (kind, c)
+        One.close()
+    M.close()
