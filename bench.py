@@ -177,7 +177,8 @@ def setup(name, device, dtype_code, level=None):
         raw = lambda l, c, xp, yp, sp: M.p2_apply_timed(l, c, xp, yp, sp, 0, 0, 0)
         timed = M.p2_apply_timed
     else:
-        kernel = "k_interior2d" if coarse.dim == 2 else "apply3d"
+        # 2D native fp64 takes a thread per point at any size
+        kernel = "apply3d" if coarse.dim == 3 else "Direct2" if dtype_code == H.F64_IEEE else "k_interior2d"
         raw, timed = M.apply_raw, M.apply_timed
     return dict(M=M, L=L, ns=ns, ng=ng, xs=xs, ys=ys, smap=smap, x_global=x, coarse=coarse,
                 interior=interior, elem=4 if dtype_code == H.F32 else 8, code=dtype_code, launches=launches,

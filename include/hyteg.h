@@ -147,11 +147,11 @@ int hyteg_dof_map(const hyteg_mesh* mesh, int level, int64_t* global_id);
 
 /* y = A x on refinement level `level` (Sec. 5.1 "apply"): A is the P1
  * stiffness matrix of the refined mesh with Dirichlet identity rows when the
- * mesh was created with HYTEG_BC_DIRICHLET.  Launches the macro-interior
- * stencil kernel (Sec. 5.2 for the 2D 7-point case; 15 points in 3D) and the
- * interface kernel, which completes the DoFs on macro vertices, edges and
- * faces by summing the contributions of every incident macro in ascending
- * macro order and writing the sum into every copy.
+ * mesh was created with HYTEG_BC_DIRICHLET.  One launch sweeps the macro
+ * interiors (Sec. 5.2 for the 2D 7-point case; 15 points in 3D) and completes
+ * the DoFs on macro vertices, edges and faces by summing the contributions of
+ * every incident macro in ascending macro order and writing the sum into every
+ * copy.
  *   dtype   HYTEG_F64, HYTEG_F32 or HYTEG_F64_IEEE (element type of x and y)
  *   x       device, [n_slots] in slot layout, copies consistent; read only
  *   y       device, [n_slots]; every slot is written; must not overlap x
@@ -192,10 +192,9 @@ int hyteg_apply_batch(const hyteg_mesh* const* meshes, const int* levels, int dt
                       void* const* ys, int count, void* stream);
 
 /* hyteg_apply with CUDA events (cudaEvent_t as void*, each may be NULL)
- * recorded on `stream` before the macro-interior kernel (ev_begin), between
- * it and the interface kernel (ev_mid) and after the interface kernel
- * (ev_end), so a caller can time each kernel on the launching stream.  The
- * events must have been created by the caller on the mesh's device.
+ * recorded on `stream` before its launch (ev_begin) and after it (ev_mid, then
+ * ev_end: the launch holds the interface step, nothing lies between the two).
+ * The events must have been created by the caller on the mesh's device.
  * Errors as hyteg_apply. */
 int hyteg_apply_timed(const hyteg_mesh* mesh, int level, int dtype, const void* x, void* y,
                       void* stream, void* ev_begin, void* ev_mid, void* ev_end);

@@ -100,14 +100,14 @@ struct LevelDev {
   int2* pts3 = nullptr;
   int n_pts3 = 0;
   // 3D, large vectors, per element type (1 float-float, 2 fp32, 3 native
-  // fp64): the columns' march, and the z-ranges per macro that the autotuner
-  // picked for it (0: not tuned, two ranges)
+  // fp64): the columns' march, or
   March3Work march[4];
-  // the element types whose products walk along rows instead (rows3d.cuh), and
-  // that kernel's tiles (x0, y0, y1, z) of a macro
+  // the walk along rows (rows3d.cuh) where set, and its tiles (x0, y0, y1, z) of a
+  // macro
   bool rows3[4] = {false, false, false, false};
   int4* tiles3 = nullptr;
   int n_tiles3 = 0;
+  // z-ranges per macro that the autotuner picked for the march (0: not tuned)
   int z_chunks[4] = {0, 0, 0, 0};
   // host copy of the class stencils (multigrid set-up)
   std::vector<double> st_host;
@@ -373,8 +373,7 @@ cudaError_t launch_apply2d(int dtype, const Mesh& m, const LevelDev& L, const vo
 cudaError_t launch_apply2d_batch(int dtype, const Mesh* const* meshes, const int* levels, const void* const* xs,
                                  void* const* ys, int count, cudaStream_t s);
 // 2D fused sweeps over u: out = u + omega dinv (b - A u) (jacobi) or
-// out = b - A u; out must not overlap u.  dtype 1 (float64, float-float
-// apply) or 2 (fp32).
+// out = b - A u; out must not overlap u.  dtype 2 (fp32).
 cudaError_t launch_sweep2d(int dtype, bool jacobi, const Mesh& m, const LevelDev& L, const void* u, const void* b,
                            const void* dinv, double omega, void* out, cudaStream_t s);
 // the fp32 fused sweeps of several 2D meshes in one launch (per mesh its
@@ -415,8 +414,7 @@ cudaError_t launch_sum_copies3d(const Mesh* const* ms, const int* levels, const 
 cudaError_t launch_sum_copies(const Mesh* const* ms, const int* levels, const double* const* x, double* const* y,
                               int count, cudaStream_t s);
 
-// The launch sequence of one apply y = A x (two kernels); `ev_mid`, when not
-// null, is recorded between them.  Returns the failing step in *what.
+// One apply y = A x; `ev_mid`, when not null, is recorded after its launch.  Returns the failing step in *what.
 cudaError_t launch_apply(const Mesh& m, int level, int dtype, const void* x, void* y, cudaStream_t s,
                          cudaEvent_t ev_mid, const char** what);
 // The apply without the interface sum: every copy of an interface point holds

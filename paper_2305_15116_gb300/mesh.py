@@ -146,7 +146,7 @@ class Mesh:
     def apply_timed(self, level: int, dtype: int, x_ptr: int, y_ptr: int, stream_ptr: int,
                     ev_begin: int, ev_mid: int, ev_end: int) -> None:
         """apply_raw that also records three CUDA events (raw cudaEvent_t
-        handles) around the macro-interior and the interface kernel."""
+        handles) before and after the launch (ev_mid: with ev_end)."""
         C.check(C.lib.hyteg_apply_timed(self._h, level, dtype, ctypes.c_void_p(x_ptr), ctypes.c_void_p(y_ptr),
                                         ctypes.c_void_p(stream_ptr), ctypes.c_void_p(ev_begin),
                                         ctypes.c_void_p(ev_mid), ctypes.c_void_p(ev_end)), "hyteg_apply_timed")
