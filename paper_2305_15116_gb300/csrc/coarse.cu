@@ -95,7 +95,7 @@ struct Cycle {
   __device__ __forceinline__ void restrict_to(const CoarseLev& F, const CoarseLev& C, bool first) const {
     float* const uc = first ? C.y : nullptr;
     auto row = [&](int cell, const Pt<2>& q) {
-      return restrict_row<2, true>(F.r + (int64_t)cell * F.S, C.multinv + cell * NCLS2, q, F.n);
+      return restrict_row<2, true, false>(F.r + (int64_t)cell * F.S, C.multinv + cell * NCLS2, q, F.n);
     };
     auto put = [&](int64_t s, float v) {
       C.b[s] = v;
@@ -118,7 +118,7 @@ struct Cycle {
       q.q[0] = q.slot - (q.q[1] * (C.n + 2) - ((q.q[1] * (q.q[1] + 1)) >> 1));
       q.q[2] = 0;
       q.M = C.n + 1;
-      put((int64_t)m * C.S + q.slot, row(m, q));
+      put((int64_t)m * C.S + q.slot, restrict_row<2, true, true>(F.r + (int64_t)m * F.S, C.multinv, q, F.n));
     }
   }
   __device__ __forceinline__ void prolong(const CoarseLev& C, const CoarseLev& F, float* uf) const {

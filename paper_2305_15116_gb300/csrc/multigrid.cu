@@ -262,7 +262,7 @@ struct Restrict {
   static __device__ __forceinline__ void run(const Prm& p, int block, int nb) {
     const int nc = p.nc;
     auto row = [&](int64_t cell, const Pt<DIM>& q) {
-      return restrict_row<DIM, false>(p.rf + cell * p.Sf, p.multinv + cell * Lat<DIM>::NCLS, q, 2 * nc);
+      return restrict_row<DIM, false, false>(p.rf + cell * p.Sf, p.multinv + cell * Lat<DIM>::NCLS, q, 2 * nc);
     };
     auto put = [&](int64_t s, T v) {
       p.bc[s] = v;
@@ -289,7 +289,7 @@ struct Restrict {
       q.set(nc);
       if (!waited) pdl_wait();
       waited = true;
-      put(i, row(cell, q));
+      put(i, restrict_row<DIM, false, true>(p.rf + cell * p.Sf, p.multinv, q, 2 * nc));
     }
     if (!waited) pdl_wait();
   }
