@@ -8,6 +8,11 @@
 // stay in registers, the x-1 / x+1 neighbours come by warp shuffles.  Every
 // slice is read three times, mostly from L2, but nothing grows with n.
 //
+// What bounds it: the issue of its instructions (66 % at 13 warps per SM with 120
+// registers in float-float, 65 % at 25 warps in fp32, L1 68 %), DRAM at 15 and 21 %.
+// us per apply against the march: 6 macros level 8 228 / 264 and 69 / 113, level 9
+// 1532 / 2061 and 471 / 863; further sizes at takes_rows3 (apply3d.cu).
+//
 // Macro-interior points only (x, y, z >= 1, x + y + z < n), whose neighbours all
 // lie inside the macro: what a lane holds beyond a row's end reaches no written
 // point.  Further blocks of the launch take the interface step (iface3d.cuh).
