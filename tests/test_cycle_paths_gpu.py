@@ -56,15 +56,15 @@ def test_coarse_meshes(cuda, k, L, kind):
     np.testing.assert_allclose(got, ref, rtol=0, atol=TOL[kind] * np.abs(ref).max())
 
 
-@pytest.mark.parametrize("nu", [(3, 3), (1, 2), (0, 2)])
-@pytest.mark.parametrize("L", [2, 4])
-def test_same_bits_as_the_separate_launches(cuda, L, nu):
+@pytest.mark.parametrize("L,nu,k", [(2, (3, 3), 12), (4, (3, 3), 12), (2, (1, 2), 12), (4, (1, 2), 12), (2, (0, 2), 12),
+                                    (4, (0, 2), 12), (2, (3, 3), 46)])
+def test_same_bits_as_the_separate_launches(cuda, L, nu, k):
     """A mesh of 8 macros alone takes the coarse levels in one launch; in a group
-    with one of 288 macros, which is too large for that, it takes every level in
-    launches of its own."""
+    with one of 288 macros, too large for that, it takes the levels above 0 in
+    launches of its own, with one of 4232 macros level 0 too."""
     import torch
     import paper_2305_15116_gb300 as H
-    ms = [unit_square_mesh(k, 0.15, k) for k in (2, 12)]
+    ms = [unit_square_mesh(q, 0.15, q) for q in (2, k)]
     Ms = [H.Mesh(m.coords, m.cells).refine(L).solver_setup(L, *nu) for m in ms]
     bs, us, los = [], [], []
     for i, M in enumerate(Ms):
